@@ -320,14 +320,24 @@ def autotune(mesh, reps=5, stream=None):
 
 
 def apply_tuning(mesh, table_path=TUNING_TABLE):
-    """Apply the stored tuning-table entry of this mesh's (dim, P, Q), if any."""
+    """Apply the stored tuning-table entry of this mesh's (dim, P, Q), if any.
+    The shapes that fill the GPU differ with the mesh: an entry that names the
+    element count it was tuned on (n_elem) serves meshes within a factor of 4
+    of it, and the closest one is taken; others keep the built-in rule."""
     import json
+    import math
     import os
     if not os.path.exists(table_path):
         return None
     key = f"{mesh.info['dim']}d_P{mesh.info['P']}_Q{mesh.info['Q']}"
-    entry = json.load(open(table_path)).get(key)
-    if entry is None:
+    if mesh._desc.geom_order == 2:
+        key += "_general"
+    entries = json.load(open(table_path)).get(key)
+    if entries is None:
+        return None
+    off = lambda e: abs(math.log(mesh.info["n_elem"] / e["n_elem"])) if "n_elem" in e else 0.0
+    entry = min(entries if isinstance(entries, list) else [entries], key=off)
+    if off(entry) > math.log(4.0):
         return None
     r = _lib.TuneResult(entry["vol_epb"], entry["vol_threads"], entry["lift_epb"],
                         entry["lift_threads"], 0.0, 0.0, 0.0, 0.0)

@@ -304,6 +304,9 @@ static void free_mesh(dg_mesh_s* m) {
   cudaFree(m->hbuf);
   cudaFree(m->tbuf);
   cudaFree(m->fbuf);
+  cudaFree(m->fflux);
+  cudaFree(m->fexp);
+  cudaFree(m->eface);
   cudaFree(m->vgeo);
   cudaFree(m->vx);
   cudaFree(m->fgeo);
@@ -406,7 +409,9 @@ dg_status dg_mesh_create(const dg_mesh_desc* md, const dg_physics* ph, void* str
   m->nq = d == 2 ? md->Q * md->Q : md->Q * md->Q * md->Q;
   m->nf = d == 2 ? md->Q : md->Q * md->Q;
   m->ndof = (long long)E * m->nv * m->nm;
+  m->curved = !boxes;
   build_tables(md->P, md->Q, m->tab);
+  build_fix_tables(md->P, md->Q, m->fix);
   init_tune(m);
   Phys& p = m->phys;
   std::memset(&p, 0, sizeof(p));
@@ -440,9 +445,15 @@ dg_status dg_mesh_create(const dg_mesh_desc* md, const dg_physics* ph, void* str
   };
   alloc((void**)&m->geo, sizeof(ElemGeo) * E);
   alloc((void**)&m->faces, sizeof(int32_t) * 6 * F);
-  alloc((void**)&m->hbuf, sizeof(double) * (size_t)E * d * m->nv * m->nq);
-  alloc((void**)&m->tbuf, sizeof(double) * ntr);
-  alloc((void**)&m->fbuf, sizeof(double) * ntr);
+  alloc((void**)&m->eface, sizeof(int32_t) * 2 * d * E);
+  if (boxes) {
+    alloc((void**)&m->fflux, sizeof(double) * (size_t)F * (3 * m->nv - 2) * m->nf);
+    alloc((void**)&m->fexp, sizeof(int32_t) * (size_t)F * 3 * m->nv);
+  } else {
+    alloc((void**)&m->hbuf, sizeof(double) * (size_t)E * d * m->nv * m->nq);
+    alloc((void**)&m->tbuf, sizeof(double) * ntr);
+    alloc((void**)&m->fbuf, sizeof(double) * ntr);
+  }
   alloc((void**)&m->scratch, sizeof(double) * 64);
   alloc((void**)&m->red, sizeof(double) * RED_BLOCKS * (MAX_RESTART + 8));
   alloc((void**)&m->hdev, sizeof(double) * 4 * (MAX_RESTART + 2));
@@ -465,6 +476,15 @@ dg_status dg_mesh_create(const dg_mesh_desc* md, const dg_physics* ph, void* str
   err = cudaMemcpyAsync(m->geo, geo.data(), sizeof(ElemGeo) * E, cudaMemcpyHostToDevice, s);
   if (err == cudaSuccess)
     err = cudaMemcpyAsync(m->faces, md->faces, sizeof(int32_t) * 6 * F, cudaMemcpyHostToDevice, s);
+  std::vector<int32_t> eface((size_t)E * 2 * d);
+  for (int f = 0; f < F; ++f) {
+    const int32_t* fp = md->faces + (size_t)f * 6;
+    eface[(size_t)fp[0] * 2 * d + fp[1]] = f;
+    if (fp[2] >= 0) eface[(size_t)fp[2] * 2 * d + fp[3]] = f;
+  }
+  if (err == cudaSuccess)
+    err = cudaMemcpyAsync(m->eface, eface.data(), sizeof(int32_t) * eface.size(),
+                          cudaMemcpyHostToDevice, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) {
     free_mesh(m);

@@ -24,6 +24,22 @@ struct Tables {
   int n, q;
 };
 
+// The 1-D tables of one (P, Q) pair as 62-bit integers (dg_fix.cuh): entry c of
+// a table with exponent e is (x 2^32 + y) with x, y its balanced halves,
+// c = that / 2^(62 - e), every row's sum of magnitudes at most 2^62.
+struct FixTab {
+  int2 B[QMAX * NMAX];    // psi_k(x_q)                                  [q][k]
+  int2 DB[QMAX * NMAX];   // psi_k'(x_q)                                 [q][k]
+  int2 D[QMAX * QMAX];    // l_k'(x_q)                                   [q][k]
+  int2 Dh[QMAX * QMAX];   // w_k l_q'(x_k) / w_q                         [q][k]
+  int2 A[NMAX * QMAX];    // (M1^-1 B^T W)                               [m][q]
+  int2 lh[2][QMAX];       // l_q(-1) / w_q, l_q(+1) / w_q
+  int2 ld[2][QMAX];       // l_q'(-1) / w_q, l_q'(+1) / w_q
+  int2 dp[2][NMAX];       // psi_k'(-1), psi_k'(+1)
+  // exponents; Dh's rows sum to at most 1/2, lh's and ld's two ends to 1/4
+  int eB, eDB, eD, eDh, eA, elh, eld, edp;
+};
+
 // Physical model on the device (copy of dg_physics with derived constants).
 struct Phys {
   double gamma, gm1, Pr, Ma, Re, mu, kappa_fac, T_inf_K, beta_s, gMa2;
@@ -80,6 +96,7 @@ struct dg_mesh_s {
   int dim, P, Q, E, nv, nm, nq, nf, F;
   long long ndof;
   dg::Tables tab;
+  dg::FixTab fix;
   dg::Phys phys;
   dg::Tune tune;
   // device buffers
@@ -94,9 +111,14 @@ struct dg_mesh_s {
   double* fbeta = nullptr;      // [F] interior-penalty factor (P+1)^2 / h
   double* minv = nullptr;       // [E][nm][nm] inverse element mass matrices
   int32_t* faces = nullptr;     // [F][6]
-  double* hbuf = nullptr;       // [E][dim][nv][nq]   weighted volume fluxes
-  double* tbuf = nullptr;       // [E][2dim][(1+dim)nv][nf] face traces
-  double* fbuf = nullptr;       // [E][2dim][(1+dim)nv][nf] face fluxes to lift
+  int32_t* eface = nullptr;     // [E][2dim] face id of each local face
+  double* hbuf = nullptr;       // general elements: [E][dim][nv][nq] weighted volume fluxes
+  double* tbuf = nullptr;       // [E][2dim][(1+dim)nv][nf] face traces (general elements, and
+                                //   the preconditioner build, which allocates it)
+  double* fbuf = nullptr;       // general elements: [E][2dim][(1+dim)nv][nf] fluxes to lift
+  double* fflux = nullptr;      // axis-aligned: [F][nv][nf] normal flux along +x_r, then
+                                //   [F][2][nv-1][nf] tangential and normal symmetric flux
+  int32_t* fexp = nullptr;      // [F][3][nv] largest exponents of those three
   double* force = nullptr;      // [ndof] M^-1 B^T wJ f (nullptr when no forcing)
   double* avf = nullptr;        // [E] artificial-viscosity factor (shock capturing only)
   dg::SensorTab stab;
@@ -179,9 +201,15 @@ struct EvalArgs {
   // optional device scalars {t, beta} read by the kernels in place of t and
   // beta, so that a captured graph serves every time level and step size
   const double* dscal = nullptr;
-  bool skip_vol = false, skip_lift = false;  // autotuning times the kernels separately
+  // autotuning times the kernels separately: the faces' (general elements:
+  // volume and faces) and the volume's (general elements: lift)
+  bool skip_face = false, skip_vol = false;
 };
 dg_status launch_residual(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s);
+// the FP64 traces of Q and grad Q at u into m->tbuf (allocated at the first
+// call), with shock capturing the elements' factors into m->avf
+dg_status launch_traces(dg_mesh_s* m, const double* u, cudaStream_t s);
+void build_fix_tables(int P, int Q, FixTab& f);
 dg_status build_general_geometry(dg_mesh_s* m, const double* nodes_host, int g, cudaStream_t s);
 dg_status launch_project(dg_mesh_s* m, int what, double t, double* out, cudaStream_t s);
 // artificial-viscosity factor mu_0 S_e h_e / P of every element at u into out [E]

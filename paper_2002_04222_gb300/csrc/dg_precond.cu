@@ -1145,12 +1145,8 @@ struct BRJImpl {
                          cudaStream_t s) {
     constexpr int NV = C::NV, NM = C::NM, NQ = C::NQ, NF = C::NF;
     const int E = m->E, nb = pc->nb, ld = round_up8(nb);
-    // traces of Q and grad Q at u (residual pass fills the trace buffer)
-    EvalArgs a{};
-    a.u = u;
-    a.t = t;
-    a.out = m->w2;
-    DG_TRY(launch_residual(m, a, s));
+    // traces of Q and grad Q at u (and the artificial-viscosity factors)
+    DG_TRY(launch_traces(m, u, s));
     double* chi = m->scratch + 8;
     var_norm_kernel<<<NV, 256, 0, s>>>(u, E, NV, NM, chi);
     DG_LAUNCHED(1);

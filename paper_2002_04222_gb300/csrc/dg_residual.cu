@@ -19,6 +19,7 @@
 #include "dg_internal.h"
 #include "dg_physics.cuh"
 #include "dg_sumfact.cuh"
+#include "dg_affine.h"
 
 namespace dg {
 
@@ -108,7 +109,8 @@ template <int DIM, int P, int Q, bool CV>
 __global__ void __launch_bounds__(32 * SENSOR_WARPS) sensor_kernel(
     const __grid_constant__ SensorTab st, const __grid_constant__ Phys ph,
     const ElemGeo* __restrict__ geo, const __grid_constant__ GenGeo gg, int E,
-    const double* __restrict__ u, double* __restrict__ avf) {
+    const double* __restrict__ u, const double* __restrict__ v, const double* __restrict__ epsp,
+    double* __restrict__ avf) {
   using C = Cfg<DIM, P, Q>;
   constexpr int NV = C::NV, NM = C::NM;
   __shared__ double sA[SENSOR_WARPS][NM], sC[SENSOR_WARPS][NM];
@@ -116,14 +118,14 @@ __global__ void __launch_bounds__(32 * SENSOR_WARPS) sensor_kernel(
   const int e = blockIdx.x * SENSOR_WARPS + w;
   if (e >= E) return;  // warp-uniform; the kernel has no block-wide barrier
   const long long base = (long long)e * NV * NM;  // variable 0: density
-  for (int k = lane; k < NM; k += 32) sA[w][k] = u[base + k];
+  for (int k = lane; k < NM; k += 32) sA[w][k] = v ? fma(epsp[0], v[base + k], u[base + k]) : u[base + k];
   __syncwarp();
   sensor_element<DIM, P, Q, CV>(st, ph, geo, gg, e, sA[w], sC[w], lane, avf);
 }
 
 // ---------------------------------------------------------------- kernel 1
 template <int DIM, int P, int Q, bool CV>
-__global__ void __launch_bounds__(256) vol_kernel(const __grid_constant__ Tables tab,
+__global__ void __launch_bounds__(256) vol_trace_kernel(const __grid_constant__ Tables tab,
                                                   const __grid_constant__ Phys ph,
                                                   const ElemGeo* __restrict__ geo,
                                                   const __grid_constant__ GenGeo gg, int E,
@@ -141,7 +143,6 @@ __global__ void __launch_bounds__(256) vol_kernel(const __grid_constant__ Tables
   double* sB = sm;
   double* sD = sB + Q * N;
   double* sl = sD + Q * Q;  // lm, lp
-  double* sw = sl + 2 * Q + N * N;
   double* sU = sm + C::TAB;            // [EPB][NV][NM]
   double* sQ = sU + EPB * NV * NM;     // [EPB][NV][NQ]
   double* sG = sQ + EPB * NV * NQ;     // DIM arrays [EPB][NV][NQ]
@@ -199,11 +200,11 @@ __global__ void __launch_bounds__(256) vol_kernel(const __grid_constant__ Tables
   if (DIM == 3) contract<Q, Q, Q2, 2, Q, Q, 1, false>(sQ, sG + 2 * EPB * NV * NQ, sD, nrep);
   __syncthreads();
   // volume flux at the Gauss points
-  for (int idx = threadIdx.x; idx < EPB * NQ; idx += blockDim.x) {
-    const int eb = idx / NQ, q = idx - eb * NQ;
-    const int e = e0 + eb;
-    if (e >= E) continue;
-    if constexpr (CV) {
+  if constexpr (CV) {
+    for (int idx = threadIdx.x; idx < EPB * NQ; idx += blockDim.x) {
+      const int eb = idx / NQ, q = idx - eb * NQ;
+      const int e = e0 + eb;
+      if (e >= E) continue;
       // general element: grad = sum_r (d xi_r/dx) d_r, contravariant flux
       // w|J| sum_j (d xi_r/d x_j) H_j
       const double* gp = gg.vgeo + (long long)e * (DIM * DIM + 1) * NQ + q;
@@ -239,30 +240,6 @@ __global__ void __launch_bounds__(256) vol_kernel(const __grid_constant__ Tables
           for (int j = 0; j < DIM; ++j) a = fma(gi[r][j], H[j][vv], a);
           hb[(r * NV + vv) * NQ] = wJ * a;
         }
-      continue;
-    }
-    const ElemGeo g = geo[e];
-    int c[3];
-    grid_coords<DIM, Q>(q, c);
-    double U[NV], dU[DIM][NV], H[DIM][NV];
-    double rh[DIM];
-#pragma unroll
-    for (int r = 0; r < DIM; ++r) rh[r] = g.rh[r];
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) {
-      U[vv] = sQ[(eb * NV + vv) * NQ + q];
-#pragma unroll
-      for (int r = 0; r < DIM; ++r) dU[r][vv] = sG[((r * EPB + eb) * NV + vv) * NQ + q] * rh[r];
-    }
-    ns_volume_flux<DIM>(U, dU, ph, H, ph.avf ? ph.avf[e] : 0.0);
-    double wJ = sw[c[0]] * sw[c[1]] * (DIM == 3 ? sw[c[2]] : 1.0);
-    wJ *= g.detJ;
-    double* hb = hbuf + (long long)e * DIM * NV * NQ + q;
-#pragma unroll
-    for (int r = 0; r < DIM; ++r) {
-      const double s = wJ * rh[r];
-#pragma unroll
-      for (int vv = 0; vv < NV; ++vv) hb[(r * NV + vv) * NQ] = s * H[r][vv];
     }
   }
   // face traces of Q and grad Q by Lagrange extrapolation along the normal
@@ -347,111 +324,6 @@ __global__ void __launch_bounds__(256) vol_kernel(const __grid_constant__ Tables
     for (int k = 0; k < Q; ++k) acc = fma(lw[k], src[base + k * str], acc);
     if (fld > 0) acc *= geo[e].rh[fld - 1];
     tbuf[(long long)e * NTR + ((lf * (1 + DIM) + fld) * NV + vv) * NF + p] = acc;
-  }
-}
-
-// ---------------------------------------------------------------- kernel 2
-template <int DIM, int P, int Q>
-__global__ void __launch_bounds__(128) face_kernel(const __grid_constant__ Tables tab,
-                                                   const __grid_constant__ Phys ph,
-                                                   const ElemGeo* __restrict__ geo,
-                                                   const int32_t* __restrict__ faces, int F,
-                                                   double t, const double* __restrict__ dscal,
-                                                   const double* __restrict__ tbuf,
-                                                   double* __restrict__ fbuf) {
-  using C = Cfg<DIM, P, Q>;
-  constexpr int NV = C::NV, NF = C::NF;
-  constexpr int NTR = 2 * DIM * (1 + DIM) * NV * NF;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= F * NF) return;
-  if (dscal) t = dscal[0];
-  const int f = idx / NF, p = idx - f * NF;
-  const int eL = faces[f * 6 + 0], fL = faces[f * 6 + 1];
-  const int eR = faces[f * 6 + 2], fR = faces[f * 6 + 3], bc = faces[f * 6 + 5];
-  const int r = fL >> 1;
-  const double sgn = (fL & 1) ? 1.0 : -1.0;
-  const ElemGeo gL = geo[eL];
-  // tangential Gauss indices of the face point
-  int pt[2] = {p % Q, DIM == 3 ? p / Q : 0};
-  double x[3] = {0, 0, 0};
-  double wJf = 1.0;
-  {
-    int a = 0;
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) {
-      if (k == r) {
-        x[k] = gL.x0[k] + ((fL & 1) ? gL.h[k] : 0.0);
-      } else {
-        x[k] = gL.x0[k] + 0.5 * (tab.x[pt[a]] + 1.0) * gL.h[k];
-        wJf *= tab.w[pt[a]] * 0.5 * gL.h[k];
-        ++a;
-      }
-    }
-  }
-  double QL[NV], dQL[DIM][NV], QR[NV], dQa[DIM][NV];
-  const double* tl = tbuf + (long long)eL * NTR + (fL * (1 + DIM)) * NV * NF + p;
-#pragma unroll
-  for (int vv = 0; vv < NV; ++vv) {
-    QL[vv] = tl[vv * NF];
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) dQL[j][vv] = tl[((1 + j) * NV + vv) * NF];
-  }
-  double rmax = gL.rh[r], cfac;  // 2 / min(h_L, h_R)
-  double rhR[DIM];
-  int bctype = 0;
-  if (eR >= 0) {
-    const ElemGeo gR = geo[eR];
-    rmax = fmax(rmax, gR.rh[r]);
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) rhR[k] = gR.rh[k];
-    const double* tr = tbuf + (long long)eR * NTR + (fR * (1 + DIM)) * NV * NF + p;
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) {
-      QR[vv] = tr[vv * NF];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) dQa[j][vv] = 0.5 * (dQL[j][vv] + tr[((1 + j) * NV + vv) * NF]);
-    }
-    cfac = 0.5;
-  } else {
-    bctype = ph.bc[bc];
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) {
-      QR[vv] = 0.0;
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) dQa[j][vv] = dQL[j][vv];
-    }
-    cfac = 1.0;
-  }
-  double Hn[NV], S[DIM][NV];
-  const double beta = (double)((P + 1) * (P + 1)) * 0.5 * rmax;  // (P+1)^2 / h
-  const double mua = av_face<DIM>(ph, eL, eR, QL, QR, dQa);
-  if (r == 0)
-    numerical_flux_axis<DIM, 0>(QL, QR, bctype, x, t, dQa, sgn, beta, ph, Hn, S, mua);
-  else if (r == 1)
-    numerical_flux_axis<DIM, 1>(QL, QR, bctype, x, t, dQa, sgn, beta, ph, Hn, S, mua);
-  else
-    numerical_flux_axis<DIM, DIM - 1>(QL, QR, bctype, x, t, dQa, sgn, beta, ph, Hn, S, mua);
-  double* fl = fbuf + (long long)eL * NTR + (fL * (1 + DIM)) * NV * NF + p;
-  const double cs = ph.viscous ? cfac * ph.beta_s * wJf : 0.0;
-  double csL[DIM];
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) csL[j] = cs * gL.rh[j];
-#pragma unroll
-  for (int vv = 0; vv < NV; ++vv) {
-    fl[vv * NF] = -Hn[vv] * wJf;
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) fl[((1 + j) * NV + vv) * NF] = csL[j] * S[j][vv];
-  }
-  if (eR >= 0) {
-    double* fr = fbuf + (long long)eR * NTR + (fR * (1 + DIM)) * NV * NF + p;
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) csL[j] = cs * rhR[j];
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) {
-      fr[vv * NF] = Hn[vv] * wJf;
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) fr[((1 + j) * NV + vv) * NF] = csL[j] * S[j][vv];
-    }
   }
 }
 
@@ -597,9 +469,8 @@ __device__ __forceinline__ void bt_minv(double* sG, double* t1, double* t2, doub
 }
 
 // ---------------------------------------------------------------- kernel 3
-template <int DIM, int P, int Q, bool CV>
+template <int DIM, int P, int Q>
 __global__ void __launch_bounds__(256) lift_kernel(const __grid_constant__ Tables tab,
-                                                   const ElemGeo* __restrict__ geo,
                                                    const __grid_constant__ GenGeo gg, int E,
                                                    const double* __restrict__ hbuf,
                                                    const double* __restrict__ fbuf,
@@ -618,7 +489,6 @@ __global__ void __launch_bounds__(256) lift_kernel(const __grid_constant__ Table
   double* sB = sm;
   double* sD = sB + Q * N;
   double* sl = sD + Q * Q;
-  double* sMi = sl + 2 * Q;
   double* sH = sm + C::TAB;             // DIM arrays [EPB][NV][NQ]
   double* sG = sH + DIM * EPB * NV * NQ;  // [EPB][NV][NQ]
   double* t1 = sG + EPB * NV * NQ;
@@ -673,22 +543,14 @@ __global__ void __launch_bounds__(256) lift_kernel(const __grid_constant__ Table
     __syncthreads();
   }
   double* sR = sH;  // reuse
-  if constexpr (CV)
-    bt_only<DIM, P, Q>(sG, t1, t2, sR, sB, nrep);
-  else
-    bt_minv<DIM, P, Q>(sG, t1, t2, sR, sB, sMi, nrep);
+  bt_only<DIM, P, Q>(sG, t1, t2, sR, sB, nrep);
   for (int i = threadIdx.x; i < EPB * NV * NM; i += blockDim.x) {
     const int eb = i / (NV * NM);
     const int e = e0 + eb;
     if (e >= E) continue;
     const long long gi = (long long)e * NV * NM + (i - eb * NV * NM);
-    double R;
-    if constexpr (CV) {
-      const int m = i % NM;
-      R = dense_minv_row<NM>(gg.minv + (long long)e * NM * NM, m, sR + (i - m));
-    } else {
-      R = sR[i] * geo[e].idet;
-    }
+    const int m = i % NM;
+    double R = dense_minv_row<NM>(gg.minv + (long long)e * NM * NM, m, sR + (i - m));
     if (force) R += force[gi];
     if (r_u) {
       const double ie = epsp[1];
@@ -773,37 +635,37 @@ __global__ void __launch_bounds__(256) project_kernel(const __grid_constant__ Ta
 }
 
 // ---------------------------------------------------------------- launchers
-template <int DIM, int P, int Q, bool CV>
-static dg_status run_residual_g(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
+template <int DIM, int P, int Q>
+static dg_status run_sensor(dg_mesh_s* m, const double* u, const double* v, const double* eps,
+                            double* out, cudaStream_t s);
+
+// general elements
+template <int DIM, int P, int Q>
+static dg_status run_residual_gen(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
   using C = Cfg<DIM, P, Q>;
   const int vepb = m->tune.vol_epb, vnt = m->tune.vol_threads;
   const int lepb = m->tune.lift_epb, lnt = m->tune.lift_threads;
   const size_t vsm = sizeof(double) * C::vol_sm(vepb), lsm = sizeof(double) * C::lift_sm(lepb);
   const GenGeo gg = gen_geo(m);
-  DG_CUDA(cudaFuncSetAttribute(vol_kernel<DIM, P, Q, CV>,
+  DG_CUDA(cudaFuncSetAttribute(vol_trace_kernel<DIM, P, Q, true>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm));
-  DG_CUDA(cudaFuncSetAttribute(lift_kernel<DIM, P, Q, CV>,
+  DG_CUDA(cudaFuncSetAttribute(lift_kernel<DIM, P, Q>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
-  if (!a.skip_vol) {
+  if (!a.skip_face) {
     // (with shock capturing the volume kernel also writes the elements'
     // artificial-viscosity factors, which the face kernel reads)
-    DG_PROF(K_VOL, s, vol_kernel<DIM, P, Q, CV><<<(m->E + vepb - 1) / vepb, vnt, vsm, s>>>(
+    DG_PROF(K_VOL, s, vol_trace_kernel<DIM, P, Q, true><<<(m->E + vepb - 1) / vepb, vnt, vsm, s>>>(
         m->tab, m->phys, m->geo, gg, m->E, a.u, a.v, a.eps, m->hbuf, m->tbuf, vepb, m->stab,
         m->phys.avf ? m->avf : nullptr));
     DG_LAUNCHED(1);
     const int nfp = m->F * C::NF;
-    if constexpr (CV) {
-      DG_PROF(K_FACE, s, face_kernel_gen<DIM, P, Q><<<(nfp + 127) / 128, 128, 0, s>>>(
-          m->phys, gg, m->faces, m->F, a.t, a.dscal, m->tbuf, m->fbuf));
-    } else {
-      DG_PROF(K_FACE, s, face_kernel<DIM, P, Q><<<(nfp + 127) / 128, 128, 0, s>>>(
-          m->tab, m->phys, m->geo, m->faces, m->F, a.t, a.dscal, m->tbuf, m->fbuf));
-    }
+    DG_PROF(K_FACE, s, face_kernel_gen<DIM, P, Q><<<(nfp + 127) / 128, 128, 0, s>>>(
+        m->phys, gg, m->faces, m->F, a.t, a.dscal, m->tbuf, m->fbuf));
     DG_LAUNCHED(1);
   }
-  if (!a.skip_lift) {
-    DG_PROF(K_LIFT, s, lift_kernel<DIM, P, Q, CV><<<(m->E + lepb - 1) / lepb, lnt, lsm, s>>>(
-        m->tab, m->geo, gg, m->E, m->hbuf, m->fbuf, m->force, a.v, a.r_u, a.eps, a.alpha, a.beta,
+  if (!a.skip_vol) {
+    DG_PROF(K_LIFT, s, lift_kernel<DIM, P, Q><<<(m->E + lepb - 1) / lepb, lnt, lsm, s>>>(
+        m->tab, gg, m->E, m->hbuf, m->fbuf, m->force, a.v, a.r_u, a.eps, a.alpha, a.beta,
         a.dscal, a.out, lepb));
     DG_LAUNCHED(1);
   }
@@ -813,17 +675,66 @@ static dg_status run_residual_g(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s)
 template <int DIM, int P, int Q>
 static dg_status run_residual(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
   if (m->curved) {
-    if constexpr (has_curved<DIM, P, Q>()) return run_residual_g<DIM, P, Q, true>(m, a, s);
+    if constexpr (has_curved<DIM, P, Q>()) return run_residual_gen<DIM, P, Q>(m, a, s);
     return DG_ERR_UNSUPPORTED;
   }
-  return run_residual_g<DIM, P, Q, false>(m, a, s);
+  if (!a.skip_face && m->phys.avf) DG_TRY((run_sensor<DIM, P, Q>(m, a.u, a.v, a.eps, m->avf, s)));
+  return launch_fix<DIM, P, Q>(m, a, s);
 }
 
+// FP64 traces for the preconditioner build: its trace Jacobians are one-sided
+// differences over 1e-8 steps, so they keep the arithmetic of the blocks' own
+// FP64 state evaluation
+template <int DIM, int P, int Q, bool CV>
+static dg_status run_traces_g(dg_mesh_s* m, const double* u, cudaStream_t s) {
+  using C = Cfg<DIM, P, Q>;
+  const size_t vsm = sizeof(double) * C::vol_sm(C::EPB);
+  DG_CUDA(cudaFuncSetAttribute(vol_trace_kernel<DIM, P, Q, CV>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm));
+  DG_PROF(K_VOL, s, vol_trace_kernel<DIM, P, Q, CV><<<(m->E + C::EPB - 1) / C::EPB, C::NT, vsm, s>>>(
+      m->tab, m->phys, m->geo, gen_geo(m), m->E, u, nullptr, nullptr, m->hbuf, m->tbuf, C::EPB,
+      m->stab, m->phys.avf ? m->avf : nullptr));
+  DG_LAUNCHED(1);
+  return DG_OK;
+}
+template <int DIM, int P, int Q>
+static dg_status run_traces(dg_mesh_s* m, const double* u, cudaStream_t s) {
+  if (m->curved) {
+    if constexpr (has_curved<DIM, P, Q>()) return run_traces_g<DIM, P, Q, true>(m, u, s);
+    return DG_ERR_UNSUPPORTED;
+  }
+  return run_traces_g<DIM, P, Q, false>(m, u, s);
+}
+
+// Launch shapes before tuning.  Axis-aligned elements: blocks of about 128
+// threads (several per SM, so that one block's contractions run beside another's
+// fluxes; 16^3 P = 3 volume kernel: 270 us at 128 threads, 332 at 224) with up
+// to 256 volume points or 224 face points, halved while the grid would leave
+// SMs idle.
 template <int DIM, int P, int Q>
 static void default_tune(dg_mesh_s* m) {
   using C = Cfg<DIM, P, Q>;
-  m->tune.vol_epb = m->tune.lift_epb = C::EPB;
-  m->tune.vol_threads = m->tune.lift_threads = C::NT;
+  if (m->curved) {
+    m->tune.vol_epb = m->tune.lift_epb = C::EPB;
+    m->tune.vol_threads = m->tune.lift_threads = C::NT;
+    return;
+  }
+  auto threads = [](int points, int most) {
+    const int t = (points + 31) / 32 * 32;
+    return t < 64 ? 64 : (t > most ? most : t);
+  };
+  int epb = 256 / C::NQ > 1 ? 256 / C::NQ : 1;
+  if (DIM == 2 && epb > 8) epb = 8;
+  while (epb > 1 && (m->E + epb - 1) / epb < 2 * 152) epb /= 2;
+  m->tune.vol_epb = epb;
+  m->tune.vol_threads = threads(epb * C::NQ, C::NQ > 256 ? 256 : 128);
+  if (DIM == 3 && m->tune.vol_threads < 128) m->tune.vol_threads = 128;
+  int fe = 224 / (C::NF * DIM) > 1 ? 224 / (C::NF * DIM) : 1;
+  if (fe > 4) fe = 4;
+  while (fe > 1 && (m->F + fe * DIM - 1) / (fe * DIM) < 2 * 152) fe /= 2;
+  m->tune.lift_epb = fe;
+  m->tune.lift_threads = threads(fe * DIM * C::NF, 224);
+  if (DIM == 3 && m->tune.lift_threads < 128) m->tune.lift_threads = 128;
 }
 
 // candidate (elements per CTA, threads per CTA) launch shapes of the
@@ -868,11 +779,6 @@ static dg_status run_project(dg_mesh_s* m, int what, double t, double* out, cuda
   return run_project_g<DIM, P, Q, false>(m, what, t, out, s);
 }
 
-// (dim, P, Q) instances built into the library
-#define DG_INSTANCES(X)                                                                       \
-  X(2, 1, 3) X(2, 2, 3) X(2, 2, 4) X(2, 3, 5) X(2, 4, 6) X(2, 5, 7) X(2, 6, 8) X(3, 1, 3) \
-  X(3, 2, 4) X(3, 2, 5) X(3, 3, 5) X(3, 3, 6) X(3, 4, 6) X(3, 4, 8)
-
 bool supported_curved(int dim, int P, int Q) {
 #define DG_SUP(D_, P_, Q_) \
   if (dim == D_ && P == P_ && Q == Q_) return true;
@@ -898,27 +804,41 @@ dg_status launch_residual(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
 }
 
 template <int DIM, int P, int Q>
-static dg_status run_sensor(dg_mesh_s* m, const double* u, double* out, cudaStream_t s) {
+static dg_status run_sensor(dg_mesh_s* m, const double* u, const double* v, const double* eps,
+                            double* out, cudaStream_t s) {
   const GenGeo gg = gen_geo(m);
   const int nb = (m->E + SENSOR_WARPS - 1) / SENSOR_WARPS;
   if (m->curved) {
     if constexpr (has_curved<DIM, P, Q>()) {
       DG_PROF(K_SENSOR, s, sensor_kernel<DIM, P, Q, true><<<nb, 32 * SENSOR_WARPS, 0, s>>>(
-          m->stab, m->phys, m->geo, gg, m->E, u, out));
+          m->stab, m->phys, m->geo, gg, m->E, u, v, eps, out));
       DG_LAUNCHED(1);
       return DG_OK;
     }
     return DG_ERR_UNSUPPORTED;
   }
   DG_PROF(K_SENSOR, s, sensor_kernel<DIM, P, Q, false><<<nb, 32 * SENSOR_WARPS, 0, s>>>(
-      m->stab, m->phys, m->geo, gg, m->E, u, out));
+      m->stab, m->phys, m->geo, gg, m->E, u, v, eps, out));
   DG_LAUNCHED(1);
   return DG_OK;
 }
 
+dg_status launch_traces(dg_mesh_s* m, const double* u, cudaStream_t s) {
+  if (!m->tbuf) {
+    const size_t n = sizeof(double) * (size_t)m->E * 2 * m->dim * (1 + m->dim) * m->nv * m->nf;
+    DG_CUDA(cudaMalloc((void**)&m->tbuf, n));
+    DG_CUDA(cudaMemsetAsync(m->tbuf, 0, n, s));
+  }
+#define DG_RUN(D_, P_, Q_) \
+  if (m->dim == D_ && m->P == P_ && m->Q == Q_) return run_traces<D_, P_, Q_>(m, u, s);
+  DG_INSTANCES(DG_RUN)
+#undef DG_RUN
+  return DG_ERR_UNSUPPORTED;
+}
+
 dg_status launch_sensor(dg_mesh_s* m, const double* u, double* out, cudaStream_t s) {
 #define DG_RUN(D_, P_, Q_) \
-  if (m->dim == D_ && m->P == P_ && m->Q == Q_) return run_sensor<D_, P_, Q_>(m, u, out, s);
+  if (m->dim == D_ && m->P == P_ && m->Q == Q_) return run_sensor<D_, P_, Q_>(m, u, nullptr, nullptr, out, s);
   DG_INSTANCES(DG_RUN)
 #undef DG_RUN
   return DG_ERR_UNSUPPORTED;
@@ -945,10 +865,11 @@ static dg_status run_autotune(dg_mesh_s* m, int reps, dg_tune_result* res, cudaS
   DG_CUDA(cudaEventCreate(&e0));
   DG_CUDA(cudaEventCreate(&e1));
   const Tune keep = m->tune;
+  // general elements: volume + faces against lift; axis-aligned: volume
+  // (with the lift in it) against faces
   auto time_it = [&](bool vol) -> double {
     EvalArgs b = a;
-    b.skip_vol = !vol;
-    b.skip_lift = vol;
+    (vol == (m->curved != 0) ? b.skip_vol : b.skip_face) = true;
     run_residual<DIM, P, Q>(m, b, s);  // warm-up
     cudaEventRecord(e0, s);
     for (int r = 0; r < reps; ++r) run_residual<DIM, P, Q>(m, b, s);
@@ -958,7 +879,7 @@ static dg_status run_autotune(dg_mesh_s* m, int reps, dg_tune_result* res, cudaS
     cudaEventElapsedTime(&ms, e0, e1);
     return ms / reps;
   };
-  // volume + face kernels (the face kernel's launch is fixed and adds the same time to each);
+  run_residual<DIM, P, Q>(m, a, s);  // face data for the volume kernel
   // the shape in effect before tuning is timed too when it is not a candidate
   double best = 1e30, dflt = -1.0;
   Tune t = keep;
