@@ -12,7 +12,8 @@ LIB = os.path.join(HERE, "libdgjfnk.so")
 SOURCES = ["dg_residual.cu", "dg_precond.cu", "dg_blas.cu", "dg_capi.cu", "dg_noalloc.cu",
            "dg_learned.cu", "dg_geometry.cu", "dg_sweep.cu", "dg_diag.cu", "dg_invert.cu",
            "dg_brj_visc.cu", "dg_fixtab.cu",
-           "dg_affine_2d.cu", "dg_affine_3a.cu", "dg_affine_3b.cu", "dg_affine_3c.cu"]
+           "dg_affine_2d.cu", "dg_affine_3a.cu", "dg_affine_3b.cu", "dg_affine_3c.cu", "dg_general_a.cu",
+           "dg_general_b.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]

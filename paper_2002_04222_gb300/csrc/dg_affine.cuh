@@ -628,6 +628,80 @@ __global__ void __maxnreg__(80) face_fix_kernel(
   for (int i = tid; i < nf * 3 * NV; i += nth) fexp[(long long)f0 * 3 * NV + i] = sS[i];
 }
 
+// ------------------------------------------------------------ volume kernels' shared parts
+// Coefficients of the elements e0 .. e0+ne-1 as doubles [ne][NV][NM] in dst,
+// their largest exponent per (element, variable) in sE; sZ zeroed.  One warp
+// per (element, variable).
+template <int DIM, int P, int Q>
+__device__ __forceinline__ void load_coefficients(const double* __restrict__ u,
+                                                  const double* __restrict__ v, double eps, int e0,
+                                                  int ne, double* dst, int* sE, int* sZ) {
+  using A = Aff<DIM, P, Q>;
+  constexpr int NV = A::NV, NM = A::NM;
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int j = threadIdx.x >> 5; j < ne * NV; j += nw) {
+    const long long g = ((long long)e0 * NV + j) * NM;
+    int m = 0;
+    for (int k = lane; k < NM; k += 32) {
+      double val = u[g + k];
+      if (v) val = fma(eps, v[g + k], val);
+      dst[j * NM + k] = val;
+      m = max(m, fix_exp(val));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) {
+      sE[j] = m;
+      sZ[j] = 0;
+    }
+  }
+}
+
+// BwdTrans: directions 0, 1 (, 2) with B; coefficients in array 1 of s1, the
+// other arrays of s1 in between, the values at the Gauss points in s0
+template <int DIM, int P, int Q>
+__device__ __forceinline__ void bwd_trans(const FixTab& ft, double* s0, double* s1, int ASZ,
+                                          const int* sE, int ne) {
+  using A = Aff<DIM, P, Q>;
+  constexpr int N = A::N, NV = A::NV, N2 = A::N2, RQ = A::RQ, VP = A::VP;
+  const int tid = threadIdx.x, nth = blockDim.x;
+  i64* t1 = (i64*)(s1 + ASZ);
+  for (int idx = tid; idx < ne * NV * N * N2; idx += nth) {
+    const int ev = idx / (N * N2);
+    int bad, xh[N], xl[N];
+    const int em = fix_emax(sE[ev], bad);
+    const double* src = s1 + idx * N;
+#pragma unroll
+    for (int k = 0; k < N; ++k) fix_split(to_fix(src[k], em, 60), xh[k], xl[k]);
+    i64* o = t1 + idx * RQ;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) o[q] = fix_dot<N>(xh, xl, ft.B + q * N);
+  }
+  __syncthreads();
+  // direction 1: [ev][n2][n1][q0] -> [ev][n2][q1][q0]
+  i64* t2 = DIM == 3 ? (i64*)(s1 + 2 * ASZ) : (i64*)s0;
+  for (int idx = tid; idx < ne * NV * N2 * Q; idx += nth) {
+    const int en = idx / Q, q0 = idx - en * Q;
+    int xh[N], xl[N];
+    fix_line<N>(t1 + en * N * RQ + q0, RQ, xh, xl);
+    i64* o = t2 + en * Q * RQ + q0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) o[q * RQ] = fix_dot<N>(xh, xl, ft.B + q * N);
+  }
+  __syncthreads();
+  if constexpr (DIM == 3) {
+    for (int idx = tid; idx < ne * NV * Q * Q; idx += nth) {
+      const int ev = idx / (Q * Q), q10 = idx - ev * Q * Q;
+      const int off = (q10 / Q) * RQ + q10 % Q;
+      int xh[N], xl[N];
+      fix_line<N>(t2 + ev * N * Q * RQ + off, Q * RQ, xh, xl);
+      i64* o = (i64*)s0 + ev * VP + off;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) o[q * Q * RQ] = fix_dot<N>(xh, xl, ft.B + q * N);
+    }
+    __syncthreads();
+  }
+}
+
 // ------------------------------------------------------------ volume kernel
 // EPB elements per block; lines of one direction are one thread's work in the
 // contractions, points in the flux.  16^3 P = 3: 270 us with the lift in it
@@ -661,25 +735,8 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
   const int ne = min(EPB, E - e0);
   if (dscal) beta = dscal[1];
   const double eps = v ? epsp[0] : 0.0;
-  // coefficients (as doubles in array 1), largest exponent per (element, variable)
+  load_coefficients<DIM, P, Q>(u, v, eps, e0, ne, s1, sE, sZ);
   {
-    const int lane = tid & 31, nw = nth >> 5;
-    for (int j = tid >> 5; j < ne * NV; j += nw) {
-      const long long g = ((long long)e0 * NV + j) * NM;
-      double* dst = s1 + j * NM;
-      int m = 0;
-      for (int k = lane; k < NM; k += 32) {
-        double val = u[g + k];
-        if (v) val = fma(eps, v[g + k], val);
-        dst[k] = val;
-        m = max(m, fix_exp(val));
-      }
-      m = __reduce_max_sync(0xffffffffu, m);
-      if (lane == 0) {
-        sE[j] = m;
-        sZ[j] = 0;
-      }
-    }
     for (int j = tid; j < ne * 2 * DIM; j += nth) {
       const int eb = j / (2 * DIM), lf = j - eb * 2 * DIM;
       ElFace x;
@@ -708,45 +765,7 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
     }
     sH[j] = m;
   }
-  // BwdTrans: directions 0, 1 (, 2) with B; s1 -> array 2 -> (array 3 ->) s0
-  {
-    i64* t1 = (i64*)(s1 + ASZ);
-    for (int idx = tid; idx < ne * NV * N * N2; idx += nth) {
-      const int ev = idx / (N * N2);
-      int bad, xh[N], xl[N];
-      const int em = fix_emax(sE[ev], bad);
-      const double* src = s1 + idx * N;
-#pragma unroll
-      for (int k = 0; k < N; ++k) fix_split(to_fix(src[k], em, 60), xh[k], xl[k]);
-      i64* o = t1 + idx * RQ;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) o[q] = fix_dot<N>(xh, xl, ft.B + q * N);
-    }
-    __syncthreads();
-    // direction 1: [ev][n2][n1][q0] -> [ev][n2][q1][q0]
-    i64* t2 = DIM == 3 ? (i64*)(s1 + 2 * ASZ) : (i64*)s0;
-    for (int idx = tid; idx < ne * NV * N2 * Q; idx += nth) {
-      const int en = idx / Q, q0 = idx - en * Q;
-      int xh[N], xl[N];
-      fix_line<N>(t1 + en * N * RQ + q0, RQ, xh, xl);
-      i64* o = t2 + en * Q * RQ + q0;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) o[q * RQ] = fix_dot<N>(xh, xl, ft.B + q * N);
-    }
-    __syncthreads();
-    if constexpr (DIM == 3) {
-      for (int idx = tid; idx < ne * NV * Q * Q; idx += nth) {
-        const int ev = idx / (Q * Q), q10 = idx - ev * Q * Q;
-        const int off = (q10 / Q) * RQ + q10 % Q;
-        int xh[N], xl[N];
-        fix_line<N>(t2 + ev * N * Q * RQ + off, Q * RQ, xh, xl);
-        i64* o = (i64*)s0 + ev * VP + off;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) o[q * Q * RQ] = fix_dot<N>(xh, xl, ft.B + q * N);
-      }
-      __syncthreads();
-    }
-  }
+  bwd_trans<DIM, P, Q>(ft, s0, s1, ASZ, sE, ne);
   const int seQ = -1022 - 60 + DIM * ft.eB;
   // reference derivatives along every direction, as doubles
   for (int idx = tid; idx < DIM * ne * NV * LQ; idx += nth) {
@@ -829,7 +848,7 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
       u64 used = 0;
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        i64 hi = 0, mid = 0;
+        i64 hi = 0, mid = FIX_HALF;
 #pragma unroll
         for (int k = 0; k < Q; ++k) {
           const int2 c = ft.Dh[q * Q + k];

@@ -16,5 +16,10 @@ namespace dg {
 
 template <int DIM, int P, int Q>
 dg_status launch_fix(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s);
+// general elements (dg_general.cuh; the instances of DG_CURVED_INSTANCES)
+template <int DIM, int P, int Q>
+dg_status launch_gen(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s);
+template <int DIM, int P, int Q>
+dg_status launch_minv_exp(dg_mesh_s* m, cudaStream_t s);
 
 }  // namespace dg

@@ -301,11 +301,10 @@ static void free_mesh(dg_mesh_s* m) {
   if (!m) return;
   cudaFree(m->geo);
   cudaFree(m->faces);
-  cudaFree(m->hbuf);
   cudaFree(m->tbuf);
-  cudaFree(m->fbuf);
   cudaFree(m->fflux);
   cudaFree(m->fexp);
+  cudaFree(m->eminv);
   cudaFree(m->eface);
   cudaFree(m->vgeo);
   cudaFree(m->vx);
@@ -435,7 +434,6 @@ dg_status dg_mesh_create(const dg_mesh_desc* md, const dg_physics* ph, void* str
     p.bc[i] = ph->bc[i];
   }
   const size_t nd = (size_t)m->ndof;
-  const size_t ntr = (size_t)E * 2 * d * (1 + d) * m->nv * m->nf;
   cudaError_t err = cudaSuccess;
   // every workspace starts zeroed: no kernel result may depend on what an
   // earlier allocation left in the memory
@@ -450,9 +448,10 @@ dg_status dg_mesh_create(const dg_mesh_desc* md, const dg_physics* ph, void* str
     alloc((void**)&m->fflux, sizeof(double) * (size_t)F * (3 * m->nv - 2) * m->nf);
     alloc((void**)&m->fexp, sizeof(int32_t) * (size_t)F * 3 * m->nv);
   } else {
-    alloc((void**)&m->hbuf, sizeof(double) * (size_t)E * d * m->nv * m->nq);
-    alloc((void**)&m->tbuf, sizeof(double) * ntr);
-    alloc((void**)&m->fbuf, sizeof(double) * ntr);
+    const size_t sides = (size_t)E * 2 * d * 2;
+    alloc((void**)&m->fflux, sizeof(double) * ((size_t)F * m->nv + sides * (m->nv - 1)) * m->nf);
+    alloc((void**)&m->fexp, sizeof(int32_t) * ((size_t)F + sides) * m->nv);
+    alloc((void**)&m->eminv, sizeof(int32_t) * (size_t)E * m->nm);
   }
   alloc((void**)&m->scratch, sizeof(double) * 64);
   alloc((void**)&m->red, sizeof(double) * RED_BLOCKS * (MAX_RESTART + 8));
@@ -493,6 +492,7 @@ dg_status dg_mesh_create(const dg_mesh_desc* md, const dg_physics* ph, void* str
   if (!boxes) {
     m->curved = 1;
     dg_status st = build_general_geometry(m, md->nodes, md->geom_order, s);
+    if (st == DG_OK) st = build_minv_exponents(m, s);
     if (st != DG_OK) {
       free_mesh(m);
       return st;

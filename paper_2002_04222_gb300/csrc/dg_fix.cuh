@@ -37,6 +37,16 @@ __device__ __forceinline__ i64 mul_wide(int a, int b) {
   return d;
 }
 
+// half a unit of a product's result, in the middle accumulator: without it
+// every contraction rounds down, and M^-1 turns the common half unit into the
+// largest error of the residual
+constexpr i64 FIX_HALF = 1ll << 29;
+
+// x / 2^sh to the nearest
+__device__ __forceinline__ i64 fix_shift(i64 x, int sh) {
+  return (x + ((1ll << sh) >> 1)) >> sh;
+}
+
 // biased exponent of a double (0x7ff for infinities and NaN)
 __device__ __forceinline__ int fix_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
@@ -75,7 +85,7 @@ __device__ __forceinline__ FixScale fix_scale(double r) {
 __device__ __forceinline__ i64 fix_mul(i64 x, int rh, int rl) {
   int h, l;
   fix_split(x, h, l);
-  const i64 mid = mul_wide(l, rh) + mul_wide(h, rl);
+  const i64 mid = FIX_HALF + mul_wide(l, rh) + mul_wide(h, rl);
   return (mul_wide(h, rh) << 2) + (mid >> 30);
 }
 
@@ -115,7 +125,7 @@ __device__ __forceinline__ int fix_emax(int e, int& bad) {
 // one output of a contraction: sum_k x_k C_k / 2^62 (inputs as halves)
 template <int K>
 __device__ __forceinline__ i64 fix_dot(const int* xh, const int* xl, const int2* C) {
-  i64 hi = 0, mid = 0;
+  i64 hi = 0, mid = FIX_HALF;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     hi += mul_wide(xh[k], C[k].x);

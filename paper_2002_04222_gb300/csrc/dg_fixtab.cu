@@ -92,7 +92,7 @@ void build_fix_tables(int P, int Q, FixTab& f) {
     w[i] = 2 / ((1 - z * z) * d * d);
   }
   const auto psi = modified_polys(P);
-  std::vector<ld> B(Q * N), DB(Q * N), D(Q * Q), Dh(Q * Q), A(N * Q), lh(2 * Q), le(2 * Q), dp(2 * N);
+  std::vector<ld> B(Q * N), DB(Q * N), D(Q * Q), Dh(Q * Q), A(N * Q), BW(N * Q), lh(2 * Q), le(2 * Q), dp(2 * N);
   for (int k = 0; k < N; ++k) {
     const auto d = poly_diff(psi[k]);
     for (int q = 0; q < Q; ++q) {
@@ -157,7 +157,11 @@ void build_fix_tables(int P, int Q, FixTab& f) {
     }
   }
   for (int a = 0; a < N; ++a)
-    for (int q = 0; q < Q; ++q) A[a * Q + q] = M[a * C + N + q];
+    for (int q = 0; q < Q; ++q) {
+      A[a * Q + q] = M[a * C + N + q];
+      BW[a * Q + q] = B[q * N + a] * w[q];
+    }
+  for (int q = 0; q < Q; ++q) f.iw[q] = (double)(1 / w[q]);
   auto ends = [&](const std::vector<ld>& v) {  // largest |v(-1)| + |v(+1)| over the points
     ld big = 0;
     for (int q = 0; q < Q; ++q) big = std::max(big, std::fabs(v[q]) + std::fabs(v[Q + q]));
@@ -176,6 +180,10 @@ void build_fix_tables(int P, int Q, FixTab& f) {
   store(D.data(), Q, Q, f.eD, f.D);
   store(Dh.data(), Q, Q, f.eDh, f.Dh);
   store(A.data(), N, Q, f.eA, f.A);
+  for (int a = 0; a < N; ++a) {
+    f.aw[a] = -row_exponent(&BW[a * Q], 1, Q);
+    store(&BW[a * Q], 1, Q, -f.aw[a], f.BW + a * Q);
+  }
   for (int s = 0; s < 2; ++s) {
     store(&lh[s * Q], 1, Q, f.elh, f.lh[s]);
     store(&le[s * Q], 1, Q, f.eld, f.ld[s]);

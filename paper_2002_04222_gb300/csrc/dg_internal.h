@@ -33,11 +33,14 @@ struct FixTab {
   int2 D[QMAX * QMAX];    // l_k'(x_q)                                   [q][k]
   int2 Dh[QMAX * QMAX];   // w_k l_q'(x_k) / w_q                         [q][k]
   int2 A[NMAX * QMAX];    // (M1^-1 B^T W)                               [m][q]
+  int2 BW[NMAX * QMAX];   // 2^aw[m] B^T W, every row scaled to at most 1  [m][q]
   int2 lh[2][QMAX];       // l_q(-1) / w_q, l_q(+1) / w_q
   int2 ld[2][QMAX];       // l_q'(-1) / w_q, l_q'(+1) / w_q
   int2 dp[2][NMAX];       // psi_k'(-1), psi_k'(+1)
   // exponents; Dh's rows sum to at most 1/2, lh's and ld's two ends to 1/4
   int eB, eDB, eD, eDh, eA, elh, eld, edp;
+  int aw[NMAX];
+  double iw[QMAX];        // 1 / w_q
 };
 
 // Physical model on the device (copy of dg_physics with derived constants).
@@ -112,13 +115,14 @@ struct dg_mesh_s {
   double* minv = nullptr;       // [E][nm][nm] inverse element mass matrices
   int32_t* faces = nullptr;     // [F][6]
   int32_t* eface = nullptr;     // [E][2dim] face id of each local face
-  double* hbuf = nullptr;       // general elements: [E][dim][nv][nq] weighted volume fluxes
-  double* tbuf = nullptr;       // [E][2dim][(1+dim)nv][nf] face traces (general elements, and
-                                //   the preconditioner build, which allocates it)
-  double* fbuf = nullptr;       // general elements: [E][2dim][(1+dim)nv][nf] fluxes to lift
+  double* tbuf = nullptr;       // [E][2dim][(1+dim)nv][nf] face traces of the preconditioner
+                                //   build, which allocates it
   double* fflux = nullptr;      // axis-aligned: [F][nv][nf] normal flux along +x_r, then
-                                //   [F][2][nv-1][nf] tangential and normal symmetric flux
-  int32_t* fexp = nullptr;      // [F][3][nv] largest exponents of those three
+                                //   [F][2][nv-1][nf] tangential and normal symmetric flux;
+                                // general: [F][nv][nf], then [E][2dim][2][nv-1][nf]
+  int32_t* fexp = nullptr;      // largest exponents of those: [F][3][nv]; general elements
+                                //   [F][nv], then [E][2dim][2][nv]
+  int32_t* eminv = nullptr;     // general: [E][nm] exponents of minv's (scaled) row sums
   double* force = nullptr;      // [ndof] M^-1 B^T wJ f (nullptr when no forcing)
   double* avf = nullptr;        // [E] artificial-viscosity factor (shock capturing only)
   dg::SensorTab stab;
@@ -201,8 +205,7 @@ struct EvalArgs {
   // optional device scalars {t, beta} read by the kernels in place of t and
   // beta, so that a captured graph serves every time level and step size
   const double* dscal = nullptr;
-  // autotuning times the kernels separately: the faces' (general elements:
-  // volume and faces) and the volume's (general elements: lift)
+  // autotuning times the faces' and the volume's kernel separately
   bool skip_face = false, skip_vol = false;
 };
 dg_status launch_residual(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s);
@@ -210,6 +213,7 @@ dg_status launch_residual(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s);
 // call), with shock capturing the elements' factors into m->avf
 dg_status launch_traces(dg_mesh_s* m, const double* u, cudaStream_t s);
 void build_fix_tables(int P, int Q, FixTab& f);
+dg_status build_minv_exponents(dg_mesh_s* m, cudaStream_t s);  // m->eminv from m->minv
 dg_status build_general_geometry(dg_mesh_s* m, const double* nodes_host, int g, cudaStream_t s);
 dg_status launch_project(dg_mesh_s* m, int what, double t, double* out, cudaStream_t s);
 // artificial-viscosity factor mu_0 S_e h_e / P of every element at u into out [E]

@@ -125,20 +125,14 @@ __global__ void __launch_bounds__(32 * SENSOR_WARPS) sensor_kernel(
 
 // ---------------------------------------------------------------- kernel 1
 template <int DIM, int P, int Q, bool CV>
-__global__ void __launch_bounds__(256) vol_trace_kernel(const __grid_constant__ Tables tab,
-                                                  const __grid_constant__ Phys ph,
-                                                  const ElemGeo* __restrict__ geo,
-                                                  const __grid_constant__ GenGeo gg, int E,
-                                                  const double* __restrict__ u,
-                                                  const double* __restrict__ v,
-                                                  const double* __restrict__ epsp,
-                                                  double* __restrict__ hbuf,
-                                                  double* __restrict__ tbuf, const int EPB,
-                                                  const __grid_constant__ SensorTab st,
-                                                  double* __restrict__ avf_out) {
+__global__ void __launch_bounds__(256) trace_kernel(const __grid_constant__ Tables tab,
+                                                    const ElemGeo* __restrict__ geo,
+                                                    const __grid_constant__ GenGeo gg, int E,
+                                                    const double* __restrict__ u,
+                                                    double* __restrict__ tbuf) {
   using C = Cfg<DIM, P, Q>;
   constexpr int N = C::N, NV = C::NV, NM = C::NM, NQ = C::NQ, NF = C::NF;
-  constexpr int Q2 = C::Q2, N2 = C::N2;
+  constexpr int Q2 = C::Q2, N2 = C::N2, EPB = C::EPB;
   extern __shared__ double sm[];
   double* sB = sm;
   double* sD = sB + Q * N;
@@ -151,34 +145,11 @@ __global__ void __launch_bounds__(256) vol_trace_kernel(const __grid_constant__ 
   const int nrep = EPB * NV;
 
   stage_tables<DIM, P, Q>(tab, sm);
-  const double eps = v ? epsp[0] : 0.0;
   for (int i = threadIdx.x; i < EPB * NV * NM; i += blockDim.x) {
     const int eb = i / (NV * NM);
-    const long long g = (long long)(e0 + eb) * NV * NM + (i - eb * NV * NM);
-    double val = 0.0;
-    if (e0 + eb < E) {
-      val = u[g];
-      if (v) val = fma(eps, v[g], val);
-    }
-    sU[i] = val;
+    sU[i] = e0 + eb < E ? u[(long long)e0 * NV * NM + i] : 0.0;
   }
   __syncthreads();
-  if (avf_out) {
-    // shock capturing: the factor of each element at the evaluated state, one
-    // warp per element, the density coefficients copied to scratch in sQ
-    // (free until BwdTrans); the volume flux below and the face kernel read it
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int eb = wp; eb < EPB; eb += nw) {
-      if (e0 + eb >= E) continue;  // warp-uniform
-      double* A = sQ + (long long)eb * NV * NQ;
-      double* Bs = A + NM;
-      for (int k = lane; k < NM; k += 32) A[k] = sU[eb * NV * NM + k];
-      __syncwarp();
-      sensor_element<DIM, P, Q, CV>(st, ph, geo, gg, e0 + eb, A, Bs, lane, avf_out);
-      __syncwarp();
-    }
-    __syncthreads();
-  }
   // BwdTrans: contract direction 0, 1 (, 2) with B
   if (DIM == 2) {
     contract<N, N, 1, 0, Q, N, 1, false>(sU, sT, sB, nrep);
@@ -199,49 +170,6 @@ __global__ void __launch_bounds__(256) vol_trace_kernel(const __grid_constant__ 
   contract<Q, Q, Q2, 1, Q, Q, 1, false>(sQ, sG + EPB * NV * NQ, sD, nrep);
   if (DIM == 3) contract<Q, Q, Q2, 2, Q, Q, 1, false>(sQ, sG + 2 * EPB * NV * NQ, sD, nrep);
   __syncthreads();
-  // volume flux at the Gauss points
-  if constexpr (CV) {
-    for (int idx = threadIdx.x; idx < EPB * NQ; idx += blockDim.x) {
-      const int eb = idx / NQ, q = idx - eb * NQ;
-      const int e = e0 + eb;
-      if (e >= E) continue;
-      // general element: grad = sum_r (d xi_r/dx) d_r, contravariant flux
-      // w|J| sum_j (d xi_r/d x_j) H_j
-      const double* gp = gg.vgeo + (long long)e * (DIM * DIM + 1) * NQ + q;
-      double gi[DIM][DIM];
-#pragma unroll
-      for (int r = 0; r < DIM; ++r)
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) gi[r][j] = gp[(r * DIM + j) * NQ];
-      const double wJ = gp[DIM * DIM * NQ];
-      double U[NV], dU[DIM][NV], H[DIM][NV];
-#pragma unroll
-      for (int vv = 0; vv < NV; ++vv) {
-        U[vv] = sQ[(eb * NV + vv) * NQ + q];
-        double dr[DIM];
-#pragma unroll
-        for (int r = 0; r < DIM; ++r) dr[r] = sG[((r * EPB + eb) * NV + vv) * NQ + q];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) {
-          double a = 0.0;
-#pragma unroll
-          for (int r = 0; r < DIM; ++r) a = fma(gi[r][j], dr[r], a);
-          dU[j][vv] = a;
-        }
-      }
-      ns_volume_flux<DIM>(U, dU, ph, H, ph.avf ? ph.avf[e] : 0.0);
-      double* hb = hbuf + (long long)e * DIM * NV * NQ + q;
-#pragma unroll
-      for (int r = 0; r < DIM; ++r)
-#pragma unroll
-        for (int vv = 0; vv < NV; ++vv) {
-          double a = 0.0;
-#pragma unroll
-          for (int j = 0; j < DIM; ++j) a = fma(gi[r][j], H[j][vv], a);
-          hb[(r * NV + vv) * NQ] = wJ * a;
-        }
-    }
-  }
   // face traces of Q and grad Q by Lagrange extrapolation along the normal
   constexpr int NTR = 2 * DIM * (1 + DIM) * NV * NF;
   if constexpr (CV) {
@@ -327,86 +255,6 @@ __global__ void __launch_bounds__(256) vol_trace_kernel(const __grid_constant__ 
   }
 }
 
-// general elements: one thread per face point with the owner-side normal,
-// surface weight and coordinates of the point, the face's penalty factor, and
-// each side's metric at the point for the symmetric-flux lift
-template <int DIM, int P, int Q>
-__global__ void __launch_bounds__(128) face_kernel_gen(const __grid_constant__ Phys ph,
-                                                       const __grid_constant__ GenGeo gg,
-                                                       const int32_t* __restrict__ faces, int F,
-                                                       double t, const double* __restrict__ dscal,
-                                                       const double* __restrict__ tbuf,
-                                                       double* __restrict__ fbuf) {
-  using C = Cfg<DIM, P, Q>;
-  constexpr int NV = C::NV, NF = C::NF;
-  constexpr int NTR = 2 * DIM * (1 + DIM) * NV * NF;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= F * NF) return;
-  if (dscal) t = dscal[0];
-  const int f = idx / NF, p = idx - f * NF;
-  const int eL = faces[f * 6 + 0], fL = faces[f * 6 + 1];
-  const int eR = faces[f * 6 + 2], fR = faces[f * 6 + 3], bc = faces[f * 6 + 5];
-  const double* fd = gg.fdat + (long long)f * (2 * DIM + 1) * NF + p;
-  double n[DIM], x[3] = {0, 0, 0};
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) {
-    n[j] = fd[j * NF];
-    x[j] = fd[(DIM + 1 + j) * NF];
-  }
-  const double wJf = fd[DIM * NF];
-  double QL[NV], QR[NV], dQa[DIM][NV];
-  const double* tl = tbuf + (long long)eL * NTR + (fL * (1 + DIM)) * NV * NF + p;
-#pragma unroll
-  for (int vv = 0; vv < NV; ++vv) {
-    QL[vv] = tl[vv * NF];
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) dQa[j][vv] = tl[((1 + j) * NV + vv) * NF];
-  }
-  int bctype = 0;
-  double cfac = 1.0;
-  if (eR >= 0) {
-    const double* tr = tbuf + (long long)eR * NTR + (fR * (1 + DIM)) * NV * NF + p;
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) {
-      QR[vv] = tr[vv * NF];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) dQa[j][vv] = 0.5 * (dQa[j][vv] + tr[((1 + j) * NV + vv) * NF]);
-    }
-    cfac = 0.5;
-  } else {
-    bctype = ph.bc[bc];
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) QR[vv] = 0.0;
-  }
-  double Hn[NV], S[DIM][NV];
-  numerical_flux_n<DIM>(QL, QR, bctype, x, t, dQa, n, gg.fbeta[f], ph, Hn, S,
-                        av_face<DIM>(ph, eL, eR, QL, QR, dQa));
-  const double cs = ph.viscous ? cfac * ph.beta_s * wJf : 0.0;
-#pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    const int e = side == 0 ? eL : eR, lf = side == 0 ? fL : fR;
-    if (e < 0) break;
-    const double* gp = gg.fgeo + ((long long)e * 2 * DIM + lf) * DIM * DIM * NF + p;
-    double* fo = fbuf + (long long)e * NTR + (lf * (1 + DIM)) * NV * NF + p;
-    const double sg = side == 0 ? -wJf : wJf;
-#pragma unroll
-    for (int vv = 0; vv < NV; ++vv) fo[vv * NF] = sg * Hn[vv];
-#pragma unroll
-    for (int r = 0; r < DIM; ++r) {
-      double gr[DIM];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) gr[j] = cs * gp[(r * DIM + j) * NF];
-#pragma unroll
-      for (int vv = 0; vv < NV; ++vv) {
-        double a = 0.0;
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) a = fma(gr[j], S[j][vv], a);
-        fo[((1 + r) * NV + vv) * NF] = a;
-      }
-    }
-  }
-}
-
 // B^T on G [EPB][NV][NQ] -> result in R [EPB][NV][NM] (general elements: the
 // dense inverse mass matrix is applied by the caller)
 template <int DIM, int P, int Q>
@@ -466,99 +314,6 @@ __device__ __forceinline__ void bt_minv(double* sG, double* t1, double* t2, doub
     contract<N, N, N2, 2, N, N, 1, false>(t1, sR, sMi, nrep);
   }
   __syncthreads();
-}
-
-// ---------------------------------------------------------------- kernel 3
-template <int DIM, int P, int Q>
-__global__ void __launch_bounds__(256) lift_kernel(const __grid_constant__ Tables tab,
-                                                   const __grid_constant__ GenGeo gg, int E,
-                                                   const double* __restrict__ hbuf,
-                                                   const double* __restrict__ fbuf,
-                                                   const double* __restrict__ force,
-                                                   const double* __restrict__ v,
-                                                   const double* __restrict__ r_u,
-                                                   const double* __restrict__ epsp, double alpha,
-                                                   double beta, const double* __restrict__ dscal,
-                                                   double* __restrict__ out, const int EPB) {
-  if (dscal) beta = dscal[1];
-  using C = Cfg<DIM, P, Q>;
-  constexpr int N = C::N, NV = C::NV, NM = C::NM, NQ = C::NQ, NF = C::NF;
-  constexpr int Q2 = C::Q2;
-  constexpr int NTR = 2 * DIM * (1 + DIM) * NV * NF;
-  extern __shared__ double sm[];
-  double* sB = sm;
-  double* sD = sB + Q * N;
-  double* sl = sD + Q * Q;
-  double* sH = sm + C::TAB;             // DIM arrays [EPB][NV][NQ]
-  double* sG = sH + DIM * EPB * NV * NQ;  // [EPB][NV][NQ]
-  double* t1 = sG + EPB * NV * NQ;
-  double* t2 = t1 + EPB * NV * NQ;
-  const int e0 = blockIdx.x * EPB;
-  const int nrep = EPB * NV;
-  stage_tables<DIM, P, Q>(tab, sm);
-  for (int i = threadIdx.x; i < EPB * DIM * NV * NQ; i += blockDim.x) {
-    const int eb = i / (DIM * NV * NQ), rem = i - eb * DIM * NV * NQ;
-    const int r = rem / (NV * NQ), o = rem - r * NV * NQ;
-    sH[(r * EPB + eb) * NV * NQ + o] =
-        e0 + eb < E ? hbuf[(long long)(e0 + eb) * DIM * NV * NQ + rem] : 0.0;
-  }
-  __syncthreads();
-  // J^T: spread the face fluxes of the 2*DIM faces onto the Gauss grid
-  for (int idx = threadIdx.x; idx < EPB * NV * NQ; idx += blockDim.x) {
-    const int eb = idx / (NV * NQ), rem = idx - eb * NV * NQ;
-    const int vv = rem / NQ, q = rem - vv * NQ;
-    const int e = e0 + eb;
-    double gsum = 0.0;
-    double hs[DIM];
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) hs[j] = 0.0;
-    if (e < E) {
-      int c[3];
-      grid_coords<DIM, Q>(q, c);
-      const double* fb = fbuf + (long long)e * NTR;
-#pragma unroll
-      for (int r = 0; r < DIM; ++r) {
-        const int p = face_point<DIM, Q>(c, r);
-        const double am = sl[c[r]], ap = sl[Q + c[r]];
-        const double* fm = fb + ((2 * r) * (1 + DIM) * NV + vv) * NF + p;
-        const double* fp = fb + ((2 * r + 1) * (1 + DIM) * NV + vv) * NF + p;
-        gsum = fma(am, fm[0], fma(ap, fp[0], gsum));
-#pragma unroll
-        for (int j = 0; j < DIM; ++j)
-          hs[j] = fma(am, fm[(1 + j) * NV * NF], fma(ap, fp[(1 + j) * NV * NF], hs[j]));
-      }
-    }
-    sG[idx] = gsum;
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) sH[j * EPB * NV * NQ + idx] += hs[j];
-  }
-  __syncthreads();
-  // G += sum_j D_j^T H_j
-  contract<Q, Q, Q2, 0, Q, 1, Q, true>(sH, sG, sD, nrep);
-  __syncthreads();
-  contract<Q, Q, Q2, 1, Q, 1, Q, true>(sH + EPB * NV * NQ, sG, sD, nrep);
-  __syncthreads();
-  if (DIM == 3) {
-    contract<Q, Q, Q2, 2, Q, 1, Q, true>(sH + 2 * EPB * NV * NQ, sG, sD, nrep);
-    __syncthreads();
-  }
-  double* sR = sH;  // reuse
-  bt_only<DIM, P, Q>(sG, t1, t2, sR, sB, nrep);
-  for (int i = threadIdx.x; i < EPB * NV * NM; i += blockDim.x) {
-    const int eb = i / (NV * NM);
-    const int e = e0 + eb;
-    if (e >= E) continue;
-    const long long gi = (long long)e * NV * NM + (i - eb * NV * NM);
-    const int m = i % NM;
-    double R = dense_minv_row<NM>(gg.minv + (long long)e * NM * NM, m, sR + (i - m));
-    if (force) R += force[gi];
-    if (r_u) {
-      const double ie = epsp[1];
-      R = (R - r_u[gi]) * ie * beta;
-      if (alpha != 0.0) R = fma(alpha, v[gi], R);
-    }
-    out[gi] = R;
-  }
 }
 
 // L2 projection of the analytic field (what = 0) or of the forcing (what = 1)
@@ -639,46 +394,14 @@ template <int DIM, int P, int Q>
 static dg_status run_sensor(dg_mesh_s* m, const double* u, const double* v, const double* eps,
                             double* out, cudaStream_t s);
 
-// general elements
-template <int DIM, int P, int Q>
-static dg_status run_residual_gen(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
-  using C = Cfg<DIM, P, Q>;
-  const int vepb = m->tune.vol_epb, vnt = m->tune.vol_threads;
-  const int lepb = m->tune.lift_epb, lnt = m->tune.lift_threads;
-  const size_t vsm = sizeof(double) * C::vol_sm(vepb), lsm = sizeof(double) * C::lift_sm(lepb);
-  const GenGeo gg = gen_geo(m);
-  DG_CUDA(cudaFuncSetAttribute(vol_trace_kernel<DIM, P, Q, true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm));
-  DG_CUDA(cudaFuncSetAttribute(lift_kernel<DIM, P, Q>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
-  if (!a.skip_face) {
-    // (with shock capturing the volume kernel also writes the elements'
-    // artificial-viscosity factors, which the face kernel reads)
-    DG_PROF(K_VOL, s, vol_trace_kernel<DIM, P, Q, true><<<(m->E + vepb - 1) / vepb, vnt, vsm, s>>>(
-        m->tab, m->phys, m->geo, gg, m->E, a.u, a.v, a.eps, m->hbuf, m->tbuf, vepb, m->stab,
-        m->phys.avf ? m->avf : nullptr));
-    DG_LAUNCHED(1);
-    const int nfp = m->F * C::NF;
-    DG_PROF(K_FACE, s, face_kernel_gen<DIM, P, Q><<<(nfp + 127) / 128, 128, 0, s>>>(
-        m->phys, gg, m->faces, m->F, a.t, a.dscal, m->tbuf, m->fbuf));
-    DG_LAUNCHED(1);
-  }
-  if (!a.skip_vol) {
-    DG_PROF(K_LIFT, s, lift_kernel<DIM, P, Q><<<(m->E + lepb - 1) / lepb, lnt, lsm, s>>>(
-        m->tab, gg, m->E, m->hbuf, m->fbuf, m->force, a.v, a.r_u, a.eps, a.alpha, a.beta,
-        a.dscal, a.out, lepb));
-    DG_LAUNCHED(1);
-  }
-  return DG_OK;
-}
-
 template <int DIM, int P, int Q>
 static dg_status run_residual(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
+  // (with shock capturing the elements' artificial-viscosity factors first)
+  if (!a.skip_face && m->phys.avf) DG_TRY((run_sensor<DIM, P, Q>(m, a.u, a.v, a.eps, m->avf, s)));
   if (m->curved) {
-    if constexpr (has_curved<DIM, P, Q>()) return run_residual_gen<DIM, P, Q>(m, a, s);
+    if constexpr (has_curved<DIM, P, Q>()) return launch_gen<DIM, P, Q>(m, a, s);
     return DG_ERR_UNSUPPORTED;
   }
-  if (!a.skip_face && m->phys.avf) DG_TRY((run_sensor<DIM, P, Q>(m, a.u, a.v, a.eps, m->avf, s)));
   return launch_fix<DIM, P, Q>(m, a, s);
 }
 
@@ -688,12 +411,12 @@ static dg_status run_residual(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
 template <int DIM, int P, int Q, bool CV>
 static dg_status run_traces_g(dg_mesh_s* m, const double* u, cudaStream_t s) {
   using C = Cfg<DIM, P, Q>;
-  const size_t vsm = sizeof(double) * C::vol_sm(C::EPB);
-  DG_CUDA(cudaFuncSetAttribute(vol_trace_kernel<DIM, P, Q, CV>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm));
-  DG_PROF(K_VOL, s, vol_trace_kernel<DIM, P, Q, CV><<<(m->E + C::EPB - 1) / C::EPB, C::NT, vsm, s>>>(
-      m->tab, m->phys, m->geo, gen_geo(m), m->E, u, nullptr, nullptr, m->hbuf, m->tbuf, C::EPB,
-      m->stab, m->phys.avf ? m->avf : nullptr));
+  if (m->phys.avf) DG_TRY((run_sensor<DIM, P, Q>(m, u, nullptr, nullptr, m->avf, s)));
+  const size_t sm = sizeof(double) * C::VOL_SM;
+  DG_CUDA(cudaFuncSetAttribute(trace_kernel<DIM, P, Q, CV>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  DG_PROF(K_VOL, s, trace_kernel<DIM, P, Q, CV><<<(m->E + C::EPB - 1) / C::EPB, C::NT, sm, s>>>(
+      m->tab, m->geo, gen_geo(m), m->E, u, m->tbuf));
   DG_LAUNCHED(1);
   return DG_OK;
 }
@@ -714,11 +437,6 @@ static dg_status run_traces(dg_mesh_s* m, const double* u, cudaStream_t s) {
 template <int DIM, int P, int Q>
 static void default_tune(dg_mesh_s* m) {
   using C = Cfg<DIM, P, Q>;
-  if (m->curved) {
-    m->tune.vol_epb = m->tune.lift_epb = C::EPB;
-    m->tune.vol_threads = m->tune.lift_threads = C::NT;
-    return;
-  }
   auto threads = [](int points, int most) {
     const int t = (points + 31) / 32 * 32;
     return t < 64 ? 64 : (t > most ? most : t);
@@ -777,6 +495,14 @@ static dg_status run_project(dg_mesh_s* m, int what, double t, double* out, cuda
     return DG_ERR_UNSUPPORTED;
   }
   return run_project_g<DIM, P, Q, false>(m, what, t, out, s);
+}
+
+dg_status build_minv_exponents(dg_mesh_s* m, cudaStream_t s) {
+#define DG_RUN(D_, P_, Q_) \
+  if (m->dim == D_ && m->P == P_ && m->Q == Q_) return launch_minv_exp<D_, P_, Q_>(m, s);
+  DG_CURVED_INSTANCES(DG_RUN)
+#undef DG_RUN
+  return DG_ERR_UNSUPPORTED;
 }
 
 bool supported_curved(int dim, int P, int Q) {
@@ -865,11 +591,9 @@ static dg_status run_autotune(dg_mesh_s* m, int reps, dg_tune_result* res, cudaS
   DG_CUDA(cudaEventCreate(&e0));
   DG_CUDA(cudaEventCreate(&e1));
   const Tune keep = m->tune;
-  // general elements: volume + faces against lift; axis-aligned: volume
-  // (with the lift in it) against faces
   auto time_it = [&](bool vol) -> double {
     EvalArgs b = a;
-    (vol == (m->curved != 0) ? b.skip_vol : b.skip_face) = true;
+    (vol ? b.skip_face : b.skip_vol) = true;
     run_residual<DIM, P, Q>(m, b, s);  // warm-up
     cudaEventRecord(e0, s);
     for (int r = 0; r < reps; ++r) run_residual<DIM, P, Q>(m, b, s);
