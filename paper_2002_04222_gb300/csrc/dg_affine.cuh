@@ -47,7 +47,7 @@ struct Aff {
   static constexpr int FY = imax(4 * NV * NT, DIM == 3 ? KK * NV * NF : 0);
   // shared memory in bytes of `e` elements / `f` faces per block
   static constexpr size_t vol_bytes(int e) {
-    return (size_t)e * (8 * VOL_EL + 2 * DIM * 28 + 3 * NV * 4);
+    return (size_t)e * (8 * VOL_EL + 2 * DIM * 28 + 4 * NV * 4);
   }
   static constexpr size_t face_bytes(int f) { return (size_t)f * (8 * (FX + FY) + 128 + 6 * NV * 4); }
 };
@@ -730,6 +730,7 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
   int* sE = (int*)(ef + EPB * 2 * DIM);         // [EPB][NV] coefficients
   int* sH = sE + EPB * NV;                      // [EPB][NV] fluxes and face data
   int* sZ = sH + EPB * NV;                      // [EPB][NV] bits of the largest |G|
+  int* sY = sZ + EPB * NV;                      // [EPB][NV] of A along the last direction
   const int tid = threadIdx.x, nth = blockDim.x;
   const int e0 = blockIdx.x * EPB;
   const int ne = min(EPB, E - e0);
@@ -764,6 +765,7 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
       }
     }
     sH[j] = m;
+    sY[j] = 0;
   }
   bwd_trans<DIM, P, Q>(ft, s0, s1, ASZ, sE, ne);
   const int seQ = -1022 - 60 + DIM * ft.eB;
@@ -880,8 +882,12 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
   }
   // A = M1^-1 B^T W along the last direction, (the middle one,) and direction 0.
   // G is far below its bound where the volume and the faces cancel, and A's
-  // row sums (16 to 32) far above its action, so G is first shifted up to 60
-  // bits; without that the result keeps 41 bits below the fluxes' largest.
+  // row sums (16 to 32) far above its action, so every stage's input is first
+  // shifted up to 60 bits and the last one's result keeps the bits that leaves
+  // free; with one scale throughout the result kept 41 bits below the fluxes'
+  // largest, and shifting G alone left the weak form's error at 8 times FP64's
+  // (4^3 modes on 6^3 points; now at most FP64's).
+  for (int j = tid; j < ne * NV; j += nth) sE[j] = 0;
   for (int idx = tid; idx < ne * NV * LQ; idx += nth) {
     const int ev = idx / LQ, l = idx - ev * LQ;
     const int off = DIM == 3 ? l % Q + RQ * (l / Q) : l;
@@ -892,35 +898,55 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
 #pragma unroll
     for (int q = 0; q < Q; ++q) fix_split(g[q * STR] << sh, xh[q], xl[q]);
     i64* o = (i64*)s0 + ev * N * STR + off;  // [ev][m_last][...][q0]
+    u64 used = 0;
 #pragma unroll
-    for (int m = 0; m < N; ++m) o[m * STR] = fix_dot<Q>(xh, xl, ft.A + m * Q);
+    for (int m = 0; m < N; ++m) {
+      const i64 x = fix_dot<Q>(xh, xl, ft.A + m * Q);
+      used |= (u64)(x ^ (x >> 63));
+      o[m * STR] = x;
+    }
+    atomicMax(sY + ev, 64 - __clzll((i64)used));
   }
   __syncthreads();
   const i64* gl = (const i64*)s0;  // [ev][..][q0] ready for direction 0
+  int* sL = sY;                    // its bits
   if constexpr (DIM == 3) {
     i64* t1 = (i64*)s1;            // [ev][n2][n1][q0]
     for (int idx = tid; idx < ne * NV * N * Q; idx += nth) {
-      const int en = idx / Q, q0 = idx - en * Q;
+      const int en = idx / Q, q0 = idx - en * Q, ev = en / N;
+      const int sh = 60 - sY[ev];
+      const i64* g = (const i64*)s0 + en * Q * RQ + q0;
       int xh[Q], xl[Q];
-      fix_line<Q>((const i64*)s0 + en * Q * RQ + q0, RQ, xh, xl);
-      i64* o = t1 + en * N * RQ + q0;
 #pragma unroll
-      for (int m = 0; m < N; ++m) o[m * RQ] = fix_dot<Q>(xh, xl, ft.A + m * Q);
+      for (int q = 0; q < Q; ++q) fix_split(g[q * RQ] << sh, xh[q], xl[q]);
+      i64* o = t1 + en * N * RQ + q0;
+      u64 used = 0;
+#pragma unroll
+      for (int m = 0; m < N; ++m) {
+        const i64 x = fix_dot<Q>(xh, xl, ft.A + m * Q);
+        used |= (u64)(x ^ (x >> 63));
+        o[m * RQ] = x;
+      }
+      atomicMax(sE + ev, 64 - __clzll((i64)used));
     }
     __syncthreads();
     gl = t1;
+    sL = sE;
   }
   // direction 0 and the epilogue
   const double ie = r_u ? epsp[1] : 0.0;
   for (int idx = tid; idx < ne * NV * N * N2; idx += nth) {
     const int ev = idx / (N * N2);
     int bad, xh[Q], xl[Q];
-    const int se = fix_emax(sH[ev], bad) - 1022 - 58 + ft.eDh + DIM * ft.eA - (60 - sZ[ev]);
-    fix_line<Q>(gl + idx * RQ, 1, xh, xl);
+    const int sh = 60 - sL[ev];
+    const int se = fix_emax(sH[ev], bad) - 1022 - 58 + ft.eDh + DIM * ft.eA - (60 - sZ[ev]) - sh - 2 -
+                   (DIM == 3 ? 60 - sY[ev] : 0);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) fix_split(gl[idx * RQ + q] << sh, xh[q], xl[q]);
     const long long gi = (long long)e0 * NV * NM + idx * N;
 #pragma unroll
     for (int m = 0; m < N; ++m) {
-      double R = fix_to_double(fix_dot<Q>(xh, xl, ft.A + m * Q), se, bad);
+      double R = fix_to_double(fix_dot<Q, 2>(xh, xl, ft.A + m * Q), se, bad);
       if (force) R += force[gi + m];
       if (r_u) {
         R = (R - r_u[gi + m]) * ie * beta;

@@ -122,17 +122,17 @@ __device__ __forceinline__ int fix_emax(int e, int& bad) {
   return max(min(e, FIX_EBAD), FIX_EMIN);
 }
 
-// one output of a contraction: sum_k x_k C_k / 2^62 (inputs as halves)
-template <int K>
+// one output of a contraction: sum_k x_k C_k / 2^(62 - S) (inputs as halves)
+template <int K, int S = 0>
 __device__ __forceinline__ i64 fix_dot(const int* xh, const int* xl, const int2* C) {
-  i64 hi = 0, mid = FIX_HALF;
+  i64 hi = 0, mid = FIX_HALF >> S;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     hi += mul_wide(xh[k], C[k].x);
     mid += mul_wide(xh[k], C[k].y);
     mid += mul_wide(xl[k], C[k].x);
   }
-  return (hi << 2) + (mid >> 30);
+  return (hi << (2 + S)) + (mid >> (30 - S));
 }
 
 // reads K values at stride `str` as halves
