@@ -64,6 +64,21 @@ __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo
     prefetch_l2(Jo + ((long long)e * 2 * DIM + threadIdx.x) * NV * NV * NF, sizeof(TJ) * NV * NV * NF);
   else if (threadIdx.x == 2 * DIM)
     prefetch_l2(q + (long long)e * NV * NM, sizeof(double) * NV * NM);
+  // general elements: M_e^-1 in the apply precision.  Up to 64 modes it is
+  // staged in shared memory, its loads issued before the gather whose phases
+  // they overlap; larger ones are read where they are used
+  constexpr bool STAGE = CV && NM <= 64;
+  __shared__ TA sMe[STAGE ? NM * NM : 1];
+  constexpr int NME = STAGE ? (NM * NM + NTH - 1) / NTH : 1;
+  double me[NME];
+  if constexpr (STAGE) {
+    const double* Me = minv + (long long)e * NM * NM;
+#pragma unroll
+    for (int t = 0; t < NME; ++t) {
+      const int i = threadIdx.x + NTH * t;
+      me[t] = i < NM * NM ? __ldcs(Me + i) : 0.0;
+    }
+  }
   for (int i = threadIdx.x; i < Q * N; i += blockDim.x) sB[i] = (TA)tab.B[i];
   for (int i = threadIdx.x; i < N * N; i += blockDim.x) sMi[i] = (TA)tab.Minv[i];
   // gather the neighbour's face slice (modes with m_r = vertex of its face)
@@ -86,6 +101,13 @@ __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo
       val = (TA)qh[((long long)en * NV + v) * NM + mc[0] + N * (mc[1] + N * mc[2])];
     }
     cs[i] = val;
+  }
+  if constexpr (STAGE) {
+#pragma unroll
+    for (int t = 0; t < NME; ++t) {
+      const int i = threadIdx.x + NTH * t;
+      if (i < NM * NM) sMe[i] = (TA)me[t];
+    }
   }
   __syncthreads();
   // face values: contract the first tangential mode index, then the second
@@ -179,23 +201,21 @@ __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo
   }
   __syncthreads();
   if constexpr (CV) {
-    // dense inverse mass matrix of the element (symmetric)
-    // (one thread per mode m: each entry of M^-1 is read once for all variables)
+    // dense inverse mass matrix of the element (symmetric), a thread per
+    // (variable, mode): with a thread per mode, 64 of 512 threads walked 64
+    // dependent loads while the rest waited (O-grid 12x24x6 P = 3, BF16
+    // blocks: 153 us per sweep of which the block product is 64)
     const double* Me = minv + (long long)e * NM * NM;
-    for (int m = threadIdx.x; m < NM; m += blockDim.x) {
-      TA s2[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) s2[v] = (TA)0;
+    for (int i = threadIdx.x; i < NV * NM; i += blockDim.x) {
+      const int m = i % NM, v0 = i - m;
+      TA s2 = (TA)0;
+#pragma unroll 8
       for (int kk = 0; kk < NM; ++kk) {
-        const TA mk = (TA)Me[kk * NM + m];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) s2[v] += mk * L0[v * NM + kk];
+        const TA mk = STAGE ? sMe[kk * NM + m] : (TA)Me[kk * NM + m];
+        s2 += mk * L0[v0 + kk];
       }
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const long long gi = ((long long)e * NV + v) * NM + m;
-        emit(v * NM + m, q[gi] + dta * (double)s2[v]);
-      }
+      const long long gi = (long long)e * NV * NM + i;
+      emit(i, q[gi] + dta * (double)s2);
     }
     return;
   }
