@@ -287,9 +287,9 @@ dg_status dg_gmres(dg_mesh_t m, dg_precond_t p, const double* u, const double* r
  * NULL) in one static device array of DG_GMRES_NOALLOC_MAX_DOUBLES doubles
  * (16 MiB) that every GPU loading the library holds until exit; it calls no
  * cudaMalloc, cudaFree or allocating routine.  It ignores cfg->graphs, and it
- * runs the preconditioner's sweeps as plain kernel launches even when p was
- * built with graphs != 0 (capturing and instantiating a graph allocates; the
- * result is the same).  Like dg_gmres, it reads each Hessenberg column back to
+ * runs the preconditioner's sweeps as kernel launches even when p was built
+ * with graphs != 0 (capturing and instantiating a graph allocates; the result
+ * is the same).  Like dg_gmres, it reads each Hessenberg column back to
  * the host and synchronises the stream after every Arnoldi step.  It returns
  * DG_ERR_ARG when n_dof * (restart + 1 + (p ? restart : 0)) exceeds the
  * array.  The first call on each device looks up the array's device address

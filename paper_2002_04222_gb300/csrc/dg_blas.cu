@@ -1,6 +1,7 @@
 // Dense FP64 vector kernels of the Krylov/Newton layer.  Reductions use a
 // fixed grid (RED_BLOCKS blocks, fixed per-block chunks, fixed-shape trees)
 // so that every norm and dot product repeats bitwise from run to run.
+#include <cooperative_groups.h>
 #include "dg_internal.h"
 
 namespace dg {
@@ -18,6 +19,167 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   double r = sh[0];
   __syncthreads();
   return r;
+}
+
+// ---------------------------------------------------------------- short vectors
+// Up to SMALL_N entries one cluster of 8 blocks does a whole reduction or the
+// whole Gram-Schmidt tail of an Arnoldi step in one launch: the entries stay in
+// registers, warps reduce eight sums at once (9 FP64 additions instead of 40:
+// the pipe retires one warp addition per 16 clocks), the blocks' sums meet in
+// distributed shared memory in rank order.  On the 8x8 P = 2 vortex (2304
+// unknowns) the 9 launches of the tail took about 40 us.  From here on the
+// grid-wide kernels below win (8 SMs of FP64 against all).
+namespace cg = cooperative_groups;
+constexpr int CL = 8, CT = 256, CR = 8;
+constexpr long long SMALL_N = (long long)CL * CT * CR;
+
+// the warp's sums of a[0..7]; lane l with l % 4 == 0 returns that of entry
+// sum8_index(l)
+__device__ __forceinline__ int sum8_index(int lane) {
+  return ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+}
+__device__ __forceinline__ double warp_sum8(double* a, int lane) {
+#pragma unroll
+  for (int o = 16, c = 4; o >= 4; o >>= 1, c >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < c; ++j) {
+      const double give = up ? a[j] : a[j + c];
+      a[j] = (up ? a[j + c] : a[j]) + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double r = a[0];
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+  return r;
+}
+// the block's sums of a[0..7] into out[0..7] (shared memory; sw: [8 warps][8])
+__device__ __forceinline__ void block_sum8(double* a, double (*sw)[8], double* out) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const double r = warp_sum8(a, lane);
+  if ((lane & 3) == 0) sw[wp][sum8_index(lane)] = r;
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double t = 0.0;
+#pragma unroll
+    for (int k = 0; k < CT / 32; ++k) t += sw[k][threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+  __syncthreads();
+}
+
+// two classical Gram-Schmidt passes of w against V_0 .. V_{k-1}, the norm and
+// the normalisation: hd[i], hd[ld + i] the passes' coefficients, hd[2 ld] =
+// |w|^2 after them; w /= |w| unless that is 0 or not finite
+__global__ void __cluster_dims__(CL) __launch_bounds__(CT) orth_cluster_kernel(
+    const double* __restrict__ V, int k, double* __restrict__ w, int n, double* __restrict__ hd,
+    int ld) {
+  __shared__ double sw[CT / 32][8], part[3][MAX_RESTART + 8], h[MAX_RESTART + 8];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), t0 = rank * CT + threadIdx.x;
+  double x[CR];
+#pragma unroll
+  for (int r = 0; r < CR; ++r) {
+    const int i = t0 + r * CL * CT;
+    x[r] = i < n ? w[i] : 0.0;
+  }
+  for (int pass = 0; pass < 3; ++pass) {
+    const int nv = pass == 2 ? 1 : k;
+    for (int i0 = 0; i0 < nv; i0 += 8) {
+      double a[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) a[j] = 0.0;
+#pragma unroll
+      for (int r = 0; r < CR; ++r) {
+        const int i = t0 + r * CL * CT;
+        if (i < n) {
+          if (pass == 2) {
+            a[0] = fma(x[r], x[r], a[0]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if (i0 + j < nv) a[j] = fma(V[(long long)(i0 + j) * n + i], x[r], a[j]);
+          }
+        }
+      }
+      block_sum8(a, sw, part[pass] + i0);
+    }
+    cl.sync();
+    for (int i = threadIdx.x; i < nv; i += CT) {
+      double s = 0.0;
+#pragma unroll
+      for (int b = 0; b < CL; ++b) s += cl.map_shared_rank(part[pass], b)[i];
+      h[i] = s;
+      if (rank == 0) hd[pass * ld + i] = s;
+    }
+    __syncthreads();
+    if (pass == 2) break;
+#pragma unroll
+    for (int r = 0; r < CR; ++r) {
+      const int i = t0 + r * CL * CT;
+      if (i < n)
+        for (int j = 0; j < k; ++j) x[r] = fma(-h[j], V[(long long)j * n + i], x[r]);
+    }
+    __syncthreads();  // h is overwritten by the next pass
+  }
+  if (threadIdx.x == 0) {
+    const double nw = sqrt(h[0]);
+    h[1] = nw > 0.0 && isfinite(nw) ? 1.0 / nw : 0.0;
+  }
+  __syncthreads();
+  const double sc = h[1];
+#pragma unroll
+  for (int r = 0; r < CR; ++r) {
+    const int i = t0 + r * CL * CT;
+    if (i < n) w[i] = sc == 0.0 ? x[r] : fma(sc, x[r], 0.0 * x[r]);
+  }
+  cl.sync();  // no block leaves while another reads its sums
+}
+
+// out[0] = a.b, or with eps the JFNK step from |a|, |b| (eps_finish_kernel)
+__global__ void __cluster_dims__(CL) __launch_bounds__(CT) dot_cluster_kernel(
+    const double* __restrict__ a, const double* __restrict__ b, int n, int eps,
+    double* __restrict__ out) {
+  __shared__ double sw[CT / 32][8], part[8];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), t0 = rank * CT + threadIdx.x;
+  double s[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) s[j] = 0.0;
+#pragma unroll
+  for (int r = 0; r < CR; ++r) {
+    const int i = t0 + r * CL * CT;
+    if (i < n) {
+      const double x = a[i], y = b[i];
+      if (eps) {
+        s[0] = fma(x, x, s[0]);
+        s[1] = fma(y, y, s[1]);
+      } else {
+        s[0] = fma(x, y, s[0]);
+      }
+    }
+  }
+  block_sum8(s, sw, part);
+  cl.sync();
+  if (rank == 0 && threadIdx.x == 0) {
+    double p = 0.0, q = 0.0;
+#pragma unroll
+    for (int r = 0; r < CL; ++r) {
+      p += cl.map_shared_rank(part, r)[0];
+      q += cl.map_shared_rank(part, r)[1];
+    }
+    if (!eps) {
+      out[0] = p;
+    } else {
+      const double nu = sqrt(p), nv = sqrt(q);
+      const double e = nv > 0.0 ? 1.4901161193847656e-08 * (nu > 0.0 ? nu : 1.0) / nv : 0.0;
+      out[0] = e;
+      out[1] = e > 0.0 ? 1.0 / e : 0.0;
+      out[2] = nu;
+      out[3] = nv;
+    }
+  }
+  cl.sync();
 }
 
 // partial[b] = sum over chunk b of a*b  (nvec independent pairs at stride)
@@ -47,6 +209,11 @@ __global__ void __launch_bounds__(RT) finish_kernel(const double* __restrict__ p
 
 dg_status dot(const double* a, const double* b, long long n, double* partial, double* out,
               cudaStream_t s) {
+  if (n <= SMALL_N) {
+    DG_PROF(K_DOT, s, dot_cluster_kernel<<<CL, CT, 0, s>>>(a, b, (int)n, 0, out));
+    DG_LAUNCHED(1);
+    return DG_OK;
+  }
   DG_PROF(K_DOT, s, dot_partial_kernel<<<RED_BLOCKS, RT, 0, s>>>(a, b, n, partial));
   DG_PROF(K_DOT, s, finish_kernel<<<1, RT, 0, s>>>(partial, RED_BLOCKS, 1, out));
   DG_LAUNCHED(2);
@@ -184,6 +351,11 @@ __global__ void eps_finish_kernel(const double* __restrict__ partial, double* __
 
 dg_status jvp_eps(const double* u, const double* v, long long n, double* partial, double* eps,
                   cudaStream_t s) {
+  if (n <= SMALL_N) {
+    DG_PROF(K_DOT, s, dot_cluster_kernel<<<CL, CT, 0, s>>>(u, v, (int)n, 1, eps));
+    DG_LAUNCHED(1);
+    return DG_OK;
+  }
   DG_PROF(K_DOT, s, dot_partial_kernel<<<RED_BLOCKS, RT, 0, s>>>(u, u, n, partial));
   DG_PROF(K_DOT, s, dot_partial_kernel<<<RED_BLOCKS, RT, 0, s>>>(v, v, n, partial + RED_BLOCKS));
   DG_PROF(K_DOT, s, eps_finish_kernel<<<1, RT, 0, s>>>(partial, eps));
@@ -236,6 +408,24 @@ dg_status normalize_dev(double* w, const double* hsq, long long n, cudaStream_t 
   DG_PROF(K_VEC, s, normalize_dev_kernel<<<grid_for(n), 256, 0, s>>>(w, hsq, n));
   DG_LAUNCHED(1);
   return DG_OK;
+}
+
+// The Gram-Schmidt tail of an Arnoldi step: w against V_0 .. V_{k-1} twice, the
+// coefficients in hd[0..k) and hd[ld..ld+k), |w|^2 in hd[2 ld], w normalised.
+// Every solver takes it, so that they agree bit for bit.
+dg_status orthonormalise(double* w, const double* V, int k, long long n, double* partial,
+                         double* hd, int ld, cudaStream_t s) {
+  if (n <= SMALL_N) {
+    DG_PROF(K_MULTIDOT, s, orth_cluster_kernel<<<CL, CT, 0, s>>>(V, k, w, (int)n, hd, ld));
+    DG_LAUNCHED(1);
+    return DG_OK;
+  }
+  DG_TRY(multi_dot(V, k, w, n, partial, hd, s));
+  DG_TRY(multi_axpy(w, V, k, hd, n, s));
+  DG_TRY(multi_dot(V, k, w, n, partial, hd + ld, s));
+  DG_TRY(multi_axpy(w, V, k, hd + ld, n, s));
+  DG_TRY(dot(w, w, n, partial, hd + 2 * ld, s));
+  return normalize_dev(w, hd + 2 * ld, n, s);
 }
 
 }  // namespace dg

@@ -41,7 +41,9 @@ __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
 // trace Jacobians, lifted onto the face modes and multiplied by the inverse
 // mass matrix, all in the apply precision TA; emit(i, y_i) receives
 // y_e = q_e + dt_a M^-1 (...) entry by entry (i = v N_m + m).
-template <int DIM, int P, int Q, typename TA, typename TJ, bool CV, int NTH, class Emit>
+// COOP: qh is written by other blocks of the same launch, so it is read from L2.
+template <int DIM, int P, int Q, typename TA, typename TJ, bool CV, int NTH, bool COOP = false,
+          class Emit>
 __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo* __restrict__ geo,
                                                 const double* __restrict__ minv,
                                                 const TJ* __restrict__ Jo,
@@ -98,7 +100,8 @@ __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo
         mc[t0] = a % N;
         mc[t1] = a / N;
       }
-      val = (TA)qh[((long long)en * NV + v) * NM + mc[0] + N * (mc[1] + N * mc[2])];
+      const double* src = qh + ((long long)en * NV + v) * NM + mc[0] + N * (mc[1] + N * mc[2]);
+      val = (TA)(COOP ? __ldcg(src) : *src);
     }
     cs[i] = val;
   }
@@ -300,7 +303,7 @@ struct Vec16<__nv_bfloat16> {
 // The block product of element e: out_e = omega D_e^-1 y_e + (1-omega) qprev_e
 // with y_e already in shared memory (sy, nb entries); part holds split x ld
 // partial sums.
-template <typename TB>
+template <typename TB, bool COOP = false>
 __device__ __forceinline__ void diag_element(const TB* __restrict__ blocks, int nb, int ld,
                                              int split, const typename Vec16<TB>::TA* sy,
                                              typename Vec16<TB>::TA* part,
@@ -345,7 +348,9 @@ __device__ __forceinline__ void diag_element(const TB* __restrict__ blocks, int 
     TA s2 = (TA)0;
     for (int k = 0; k < split; ++k) s2 += part[k * ld + r];
     const long long gi = (long long)e * nb + r;
-    out[gi] = omega == 1.0 ? (double)s2 : omega * (double)s2 + (1.0 - omega) * qprev[gi];
+    out[gi] = omega == 1.0
+                  ? (double)s2
+                  : omega * (double)s2 + (1.0 - omega) * (COOP ? __ldcg(qprev + gi) : qprev[gi]);
   }
 }
 

@@ -630,7 +630,7 @@ static dg_status arnoldi_step_ops(dg_mesh_s* m, dg_precond_s* p, const double* u
   const double* zk = vk;
   if (p) {
     double* zz = V + (size_t)(mr + 1) * n + (size_t)k * n;
-    DG_TRY(precond_sweeps(p, vk, zz, s));
+    DG_TRY(precond_solver_apply(p, vk, zz, s));
     zk = zz;
   }
   double* w = V + (size_t)(k + 1) * n;
@@ -644,13 +644,9 @@ static dg_status arnoldi_step_ops(dg_mesh_s* m, dg_precond_s* p, const double* u
   a.dscal = dscal;
   a.out = w;
   DG_TRY(launch_residual(m, a, s));
-  DG_TRY(multi_dot(V, k + 1, w, n, m->red, hd, s));
-  DG_TRY(multi_axpy(w, V, k + 1, hd, n, s));
-  DG_TRY(multi_dot(V, k + 1, w, n, m->red, hd + (mr + 2), s));
-  DG_TRY(multi_axpy(w, V, k + 1, hd + (mr + 2), n, s));
-  DG_TRY(dot(w, w, n, m->red, hd + 2 * (mr + 2), s));
+  DG_TRY(orthonormalise(w, V, k + 1, n, m->red, hd, mr + 2, s));
   DG_CUDA(cudaMemcpyAsync(m->hhost, hd, sizeof(double) * 3 * (mr + 2), cudaMemcpyDeviceToHost, s));
-  return normalize_dev(w, hd + 2 * (mr + 2), n, s);
+  return DG_OK;
 }
 
 static constexpr size_t kMaxArnoldiGraphs = 2 * MAX_RESTART;
@@ -751,16 +747,15 @@ static dg_status gmres_impl(dg_mesh_s* m, dg_precond_s* p, const double* u, cons
         const double* zk = vk;
         if (p) {
           double* zz = Z + (size_t)k * n;
-          DG_TRY(precond_apply_impl(p, vk, zz, s));
+          if (precond_one_launch(p))
+            DG_TRY(precond_solver_apply(p, vk, zz, s));
+          else
+            DG_TRY(precond_apply_impl(p, vk, zz, s));
           zk = zz;
         }
         DG_TRY(apply_A(m, u, r_u, t, dta, zk, w, s));
         // classical Gram-Schmidt, applied twice
-        DG_TRY(multi_dot(V, k + 1, w, n, m->red, hd, s));
-        DG_TRY(multi_axpy(w, V, k + 1, hd, n, s));
-        DG_TRY(multi_dot(V, k + 1, w, n, m->red, hd + (mr + 2), s));
-        DG_TRY(multi_axpy(w, V, k + 1, hd + (mr + 2), n, s));
-        DG_TRY(dot(w, w, n, m->red, hd + 2 * (mr + 2), s));
+        DG_TRY(orthonormalise(w, V, k + 1, n, m->red, hd, mr + 2, s));
         DG_CUDA(cudaMemcpyAsync(hh, hd, sizeof(double) * 3 * (mr + 2), cudaMemcpyDeviceToHost, s));
       }
       S.iters++;
@@ -769,8 +764,6 @@ static dg_status gmres_impl(dg_mesh_s* m, dg_precond_s* p, const double* u, cons
       if (!std::isfinite(hn)) return DG_ERR_NONFINITE;
       for (int i = 0; i <= k; ++i) H[(size_t)i * mr + k] = hh[i] + hh[(mr + 2) + i];
       H[(size_t)(k + 1) * mr + k] = hn;
-      // (the graph normalised w on the device)
-      if (!use_graph && hn > 0.0) DG_TRY(axpby(w, 1.0 / hn, w, 0.0, n, s));
       for (int i = 0; i < k; ++i) {
         double t0 = cs[i] * H[(size_t)i * mr + k] + sn[i] * H[(size_t)(i + 1) * mr + k];
         H[(size_t)(i + 1) * mr + k] = -sn[i] * H[(size_t)i * mr + k] + cs[i] * H[(size_t)(i + 1) * mr + k];

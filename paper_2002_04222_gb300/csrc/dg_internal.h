@@ -253,6 +253,8 @@ dg_status newton_resid(double* N, const double* u, const double* S, const double
 dg_status set_scalars(double* d, double a, double b, cudaStream_t s);  // d[0] = a, d[1] = b
 // w = w / sqrt(*hsq) when sqrt(*hsq) > 0 (the same arithmetic as axpby(w, 1/h, w, 0))
 dg_status normalize_dev(double* w, const double* hsq, long long n, cudaStream_t s);
+dg_status orthonormalise(double* w, const double* V, int k, long long n, double* partial,
+                         double* hd, int ld, cudaStream_t s);
 void drop_arnoldi_graphs(dg_mesh_s* m);
 
 }  // namespace dg

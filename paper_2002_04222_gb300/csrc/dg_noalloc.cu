@@ -110,26 +110,21 @@ extern "C" dg_status dg_gmres_noalloc(dg_mesh_t m, dg_precond_t p, const double*
       const double* zk = vk;
       if (p) {
         double* zz = Z + (size_t)k * n;
-        // plain launches, never the graph replay: capturing and instantiating
-        // a graph allocates (precond_sweeps is what the replay runs)
-        DG_TRY(precond_sweeps(p, vk, zz, s));
+        // launches, never the graph replay: capturing and instantiating a graph
+        // allocates (this is what the replay of dg_gmres runs)
+        DG_TRY(precond_solver_apply(p, vk, zz, s));
         zk = zz;
       }
       double* w = V + (size_t)(k + 1) * n;
       DG_TRY(dg_jvp(m, u, r_u, t, zk, 1.0, -dt_a, w, s));
       S.iters++;
-      DG_TRY(multi_dot(V, k + 1, w, n, m->red, hd, s));
-      DG_TRY(multi_axpy(w, V, k + 1, hd, n, s));
-      DG_TRY(multi_dot(V, k + 1, w, n, m->red, hd + (mr + 2), s));
-      DG_TRY(multi_axpy(w, V, k + 1, hd + (mr + 2), n, s));
-      DG_TRY(dot(w, w, n, m->red, hd + 2 * (mr + 2), s));
+      DG_TRY(orthonormalise(w, V, k + 1, n, m->red, hd, mr + 2, s));
       DG_CUDA(cudaMemcpyAsync(hh, hd, sizeof(double) * 3 * (mr + 2), cudaMemcpyDeviceToHost, s));
       DG_CUDA(cudaStreamSynchronize(s));
       const double hn = std::sqrt(hh[2 * (mr + 2)]);
       if (!std::isfinite(hn)) return DG_ERR_NONFINITE;
       for (int i = 0; i <= k; ++i) H[(size_t)i * mr + k] = hh[i] + hh[(mr + 2) + i];
       H[(size_t)(k + 1) * mr + k] = hn;
-      if (hn > 0.0) DG_TRY(axpby(w, 1.0 / hn, w, 0.0, n, s));
       for (int i = 0; i < k; ++i) {
         const double t0 = cs[i] * H[(size_t)i * mr + k] + sn[i] * H[(size_t)(i + 1) * mr + k];
         H[(size_t)(i + 1) * mr + k] = -sn[i] * H[(size_t)i * mr + k] + cs[i] * H[(size_t)(i + 1) * mr + k];

@@ -1365,6 +1365,12 @@ dg_status precond_sweeps(dg_precond_s* pc, const double* q, double* out, cudaStr
   return DG_OK;
 }
 
+// (per-kernel profiling keeps the sweeps apart)
+bool precond_one_launch(const dg_precond_s* pc) { return pc->coop && !profiling_on(); }
+dg_status precond_solver_apply(dg_precond_s* pc, const double* q, double* out, cudaStream_t s) {
+  return precond_one_launch(pc) ? dispatch_coop_apply(pc, q, out, s) : precond_sweeps(pc, q, out, s);
+}
+
 static constexpr size_t kMaxGraphs = 128;
 
 void precond_drop_graphs(dg_precond_s* pc) {
@@ -1436,6 +1442,7 @@ static void free_precond(dg_precond_s* p) {
   cudaFree(p->tr);
   cudaFree(p->qh);
   cudaFree(p->qh2);
+  cudaFree(p->bar);
   cudaFree(p->y);
   cudaFree(p->work);
   cudaFree(p->jk);
@@ -1550,7 +1557,12 @@ dg_status dg_precond_build(dg_mesh_t m, const double* u, double t, double dt_a,
   if (p->gen == 0 || p->J != cfg->J || p->omega != cfg->omega || p->dt_a != dt_a ||
       p->fused != (cfg->fused != 0))
     p->gen = __atomic_add_fetch(&g_gen, 1ULL, __ATOMIC_RELAXED);
-  if (cfg->fused && !p->qh2) {
+  if (!p->bar && !full) {
+    p->coop = dispatch_coop_apply(p, nullptr, nullptr, s) == DG_OK;
+    DG_CUDA(cudaMalloc((void**)&p->bar, 2 * sizeof(unsigned long long)));
+    DG_CUDA(cudaMemset(p->bar, 0, 2 * sizeof(unsigned long long)));
+  }
+  if ((cfg->fused || p->coop) && !p->qh2) {
     DG_CUDA(cudaMalloc((void**)&p->qh2, sizeof(double) * (size_t)m->ndof));
     DG_CUDA(cudaMemset(p->qh2, 0, sizeof(double) * (size_t)m->ndof));
   }

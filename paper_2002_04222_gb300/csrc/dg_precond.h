@@ -32,7 +32,10 @@ struct dg_precond_s {
   int use_graphs = 0;
   int tc_invert = 0;      // FP32 blocks: trailing updates of the inversion on the tensor cores
   int fused = 0;          // sweeps j >= 2 as one off-diagonal + block kernel
-  double* qh2 = nullptr;  // [ndof] second iterate buffer of the fused sweeps (lazily allocated)
+  double* qh2 = nullptr;  // [ndof] second iterate buffer of the fused sweeps and of the
+                          // one-launch apply (lazily allocated)
+  int coop = 0;           // every element resident at once: the solvers apply in one launch
+  unsigned long long* bar = nullptr;  // [2] its counter and its failure mark
   // terms 4-5 of the element Jacobian (full_jacobian): per element face and
   // point, K = s wJ dH/d grad Q [k][j][l], S_own / S_nbr = c wJ dS/dQ [i][k][l]
   int full = 0;
@@ -51,6 +54,11 @@ dg_status dispatch_sweep(dg_precond_s* p, const double* qprev, const double* q, 
                          cudaStream_t s);
 // the apply as plain kernel launches on s (for capture inside a larger graph)
 dg_status precond_sweeps(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
+// the apply of the solvers: one cooperative launch where the elements fit the
+// GPU together (dg_sweep.cu; out = nullptr asks whether they do), else the above
+dg_status dispatch_coop_apply(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
+bool precond_one_launch(const dg_precond_s* p);
+dg_status precond_solver_apply(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
 void precond_drop_graphs(dg_precond_s* p);
 // in-place inversion of E blocks nb x nb (row stride ld), panel in registers
 // (dg_invert.cu); supported for nb up to 640 (FP32) / 384 (FP64)
