@@ -445,8 +445,69 @@ __global__ void __launch_bounds__(128) brj_tracejac_gen_kernel(
 // q0 per (j,a) accumulated by the types of direction 1, then q1.  The own-side
 // trace term adds, on each face, the face-slice modes (vertex mode across the
 // face) contracted over the two (one) tangential face-point directions.
+// the FP64 form of a mass-matrix row, out of line: inlined, the compiler
+// predicates its few instructions instead of branching round them and the FP64
+// pipe is as busy as before
+template <int N, typename T>
+__device__ __noinline__ T fp64_row(const double* m, const T* x, int str) {
+  double s = 0.0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) s += m[k] * (double)x[k * str];
+  return (T)s;
+}
+template <typename T>
+__device__ __noinline__ T fp64_scaled(double sc, T x, double add) {
+  return (T)__dadd_rn(__dmul_rn(sc, (double)x), add);
+}
+
+// shared-memory layout of the block assembly
+template <int DIM, int P, int Q>
+struct BlockSmem {
+  static constexpr int N = P + 1, N2 = N * N, NM = DIM == 3 ? N2 * N : N2;
+  // n1 stride of T2: N N2 values, padded (from N = 4 on) to N2 modulo 32
+  static constexpr int T2N = N * N2 + (N >= 4 ? ((N2 - N * N2) % 32 + 32) % 32 : 0);
+  static constexpr int imax(int a, int b) { return a > b ? a : b; }
+  // (the trace term uses both for the faces' Jacobians and half contractions)
+  static constexpr int T1SZ = DIM == 3 ? 6 * N2 * Q * Q : 4 * N2 * Q;
+  static constexpr int T2SZ = DIM == 3 ? imax(Q * N * T2N, 6 * N2 * Q) : 0;
+  static constexpr int XS = DIM == 3 && NM % 32 == 0 ? NM + 8 : NM;  // row stride of X and Y
+};
+
+// FP32 results of FP64 arithmetic without the FP64 pipe.  A sum of products
+// m_k x_k (m_k doubles, x_k floats) is formed in float pairs (error below 2^-42
+// of the terms' magnitudes) and rounded; where it lies too close to a rounding
+// boundary to tell on which side the FP64 sum falls, near() says so and the
+// caller takes the FP64 form, so that the result is FP64's bit for bit.  The
+// mass-matrix step of a P = 3 block is 49,000 FP64 multiply-adds, 25 blocks per
+// element, on a pipe that retires two per clock.  Entries that cancel to
+// rounding noise cannot be told and keep FP64 (6^3 elements, P = 3: 1.30 ms of
+// assembly with FP64 and the former shared-memory layouts, 0.99 with both).
+struct PairSum {
+  float s = 0.f, c = 0.f, big = 0.f;
+  __device__ __forceinline__ void add(float mh, float ml, float x) {
+    const float p = __fmul_rn(mh, x);
+    const float e = __fmaf_rn(ml, x, __fmaf_rn(mh, x, -p));
+    const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
+    const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b));
+    s = t;
+    c = __fadd_rn(c, __fadd_rn(r, e));
+    big += fabsf(p);
+  }
+  __device__ __forceinline__ float value() const { return __fadd_rn(s, c); }
+  // the pair within 2^-42 of the terms of a boundary between two floats, or
+  // out of the range where that is told apart from the value's own exponent
+  __device__ __forceinline__ bool near(float v) const {
+    const int b = __float_as_int(v), E = b & 0x7f800000;
+    const float half = __int_as_float(E - (24 << 23));  // half a unit of v
+    const float left = fabsf(__fsub_rn(c, __fsub_rn(v, s)));
+    return big != 0.f && (E < (60 << 23) || E > (250 << 23) ||
+                          (b & 0x7fffff) == 0 ||
+                          !(half - left > big * 2.3e-13f));
+  }
+};
+
 template <int DIM, int P, int Q, typename T, bool CV>
-__global__ void __launch_bounds__(256) brj_block_kernel(
+__global__ void __launch_bounds__(256, sizeof(T) == 4 && P <= 3 ? 3 : 1) brj_block_kernel(
     const __grid_constant__ Tables tab, const ElemGeo* __restrict__ geo,
     const double* __restrict__ minv, int e_begin, const T* __restrict__ W,
     const T* __restrict__ Jd, double dta, T* __restrict__ blocks, int ld) {
@@ -455,16 +516,18 @@ __global__ void __launch_bounds__(256) brj_block_kernel(
   constexpr int NW = DIM * (DIM + 1) * NV * NV;
   constexpr int JA = DIM * (DIM + 1);
   constexpr int N2 = N * N;
-  // 3-D: T1 [N2][Q*Q] per (j,a), T2 [N2*N2][Q] per type; 2-D: T1 [4][N2][Q]
-  constexpr int T1SZ = DIM == 3 ? N2 * Q * Q : 4 * N2 * Q;
-  constexpr int T2SZ = DIM == 3 ? N2 * N2 * Q : 0;
+  // 3-D: T1 [up to 6 (j,a) of a type][Q*Q][N2], T2 [Q][N n1][N m1][N2]
+  // per type; 2-D: T1 [4][N2][Q]
+  using BS = BlockSmem<DIM, P, Q>;
+  constexpr int T1SZ = BS::T1SZ, T2SZ = BS::T2SZ, T2N = BS::T2N, T2Q = N * T2N, XS = BS::XS;
   __shared__ T sB1[Q * N], sD1[Q * N];
   __shared__ double sMi[N * N];
+  __shared__ float sMh[N * N], sMl[N * N];
   extern __shared__ unsigned char smraw[];
-  T* X = reinterpret_cast<T*>(smraw);           // [NM (col n)][NM (row m)]
-  T* Y = X + NM * NM;
-  T* sW = Y + NM * NM;                          // [JA][NQ]; later the dense M^-1
-  T* T1 = sW + (CV && NM * NM > JA * NQ ? NM * NM : JA * NQ);
+  T* X = reinterpret_cast<T*>(smraw);           // [NM (col n)][XS (row m)]
+  T* Y = X + NM * XS;
+  T* sW = Y + NM * XS;                          // [JA][NQ]; later the dense M^-1, over T1 and T2 too
+  T* T1 = sW + JA * NQ;
   T* T2 = T1 + T1SZ;
   const int el = blockIdx.x, e = e_begin + el;
   const int k = blockIdx.y / NV, l = blockIdx.y % NV;
@@ -475,7 +538,11 @@ __global__ void __launch_bounds__(256) brj_block_kernel(
     for (int j = 0; j < Q; ++j) d += tab.Dq[q * Q + j] * tab.B[j * N + m];
     sD1[i] = (T)d;
   }
-  for (int i = threadIdx.x; i < N * N; i += blockDim.x) sMi[i] = tab.Minv[i];
+  for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
+    sMi[i] = tab.Minv[i];
+    sMh[i] = (float)tab.Minv[i];
+    sMl[i] = (float)(tab.Minv[i] - (double)(float)tab.Minv[i]);
+  }
   const T* We = W + (long long)el * NQ * NW;
   for (int i = threadIdx.x; i < NQ * JA; i += blockDim.x)
     sW[i] = We[(long long)(k * NV + l) * JA * NQ + i];  // contiguous slice of (k, l)
@@ -499,77 +566,102 @@ __global__ void __launch_bounds__(256) brj_block_kernel(
     }
     // one pass per factor type of direction 2 (f2, g2 in {b, d}): the (j, a)
     // of that type are contracted over q0 and q1 into T2, then q2 into X
-    for (int i = threadIdx.x; i < NM * NM; i += blockDim.x) X[i] = (T)0;
+    // (layouts: the index that neighbouring lanes walk is the fastest, N n1 and
+    // the rows of X padded so that a warp's two groups fall on different banks;
+    // the former layouts met 8-way conflicts in the last contraction.  The (j, a)
+    // of a type go through q0 together, up to six times the threads' work per
+    // barrier, and their sums over q1 stay in registers)
+    for (int i = threadIdx.x; i < NM * XS; i += blockDim.x) X[i] = (T)0;
+    __syncthreads();
+    constexpr int IT = (N2 * N * Q + 255) / 256;  // (256 threads)
     for (int type = 0; type < 4; ++type) {
-      for (int i = threadIdx.x; i < N2 * N2 * Q; i += blockDim.x) T2[i] = (T)0;
-      __syncthreads();
-      for (int ja = 0; ja < JA; ++ja) {
-        const int j = ja / (DIM + 1), a = ja % (DIM + 1);
-        if ((j == 2 ? 2 : 0) + (a == 3 ? 1 : 0) != type) continue;
+      // the c-th (j, a) of the type: j = 0, 1 (types 0, 1) or 2, a = 0..2 or 3
+      const int na = (type & 1) ? 1 : 3, count = (type & 2) ? na : 2 * na;
+      auto comb = [&](int c, int& j, int& a) {
+        j = (type & 2) ? 2 : c / na;
+        a = (type & 1) ? 3 : c % na;
+      };
+      // contract q0: T1[c][q1 + Q q2][m0 + N n0], a thread per (c, q1 q2, n0), m0 in registers
+      for (int i = threadIdx.x; i < count * Q * Q * N; i += blockDim.x) {
+        const int n0 = i % N, r = i / N, qq = r % (Q * Q), c = r / (Q * Q);
+        int j, a;
+        comb(c, j, a);
         const T* fg0 = FG + ((j == 0 ? 2 : 0) + (a == 1 ? 1 : 0)) * Q * N2;
-        const T* fg1 = FG + ((j == 1 ? 2 : 0) + (a == 2 ? 1 : 0)) * Q * N2;
-        const T* w = sW + ja * NQ;
-        // contract q0: T1[(m0 + N n0)][q1 + Q q2], a thread per (q1 q2, n0), m0 in registers
-        for (int i = threadIdx.x; i < Q * Q * N; i += blockDim.x) {
-          const int qq = i % (Q * Q), n0 = i / (Q * Q);
-          T acc[N];
+        const T* w = sW + (j * (DIM + 1) + a) * NQ;
+        T acc[N];
 #pragma unroll
-          for (int m0 = 0; m0 < N; ++m0) acc[m0] = (T)0;
+        for (int m0 = 0; m0 < N; ++m0) acc[m0] = (T)0;
 #pragma unroll
-          for (int q0 = 0; q0 < Q; ++q0) {
-            const T wv = w[q0 + Q * qq];
-            const T* fr = fg0 + q0 * N2 + N * n0;
+        for (int q0 = 0; q0 < Q; ++q0) {
+          const T wv = w[q0 + Q * qq];
+          const T* fr = fg0 + q0 * N2 + N * n0;
 #pragma unroll
-            for (int m0 = 0; m0 < N; ++m0) acc[m0] += fr[m0] * wv;
-          }
-#pragma unroll
-          for (int m0 = 0; m0 < N; ++m0) T1[(m0 + N * n0) * Q * Q + qq] = acc[m0];
+          for (int m0 = 0; m0 < N; ++m0) acc[m0] += fr[m0] * wv;
         }
-        __syncthreads();
-        // contract q1: T2[((m0 + N n0) N2 + m1 + N n1) Q + q2] +=, a thread per
-        // (mn0, q2, n1), m1 in registers
-        for (int i = threadIdx.x; i < N2 * Q * N; i += blockDim.x) {
-          const int q2 = i % Q, r = i / Q;
-          const int n1 = r % N, mn0 = r / N;
+#pragma unroll
+        for (int m0 = 0; m0 < N; ++m0) T1[(c * Q * Q + qq) * N2 + N * n0 + m0] = acc[m0];
+      }
+      __syncthreads();
+      // contract q1, a thread per (mn0, n1, q2), m1 in registers
+      T sum[IT][N];
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const int i = threadIdx.x + 256 * it;
+#pragma unroll
+        for (int m1 = 0; m1 < N; ++m1) sum[it][m1] = (T)0;
+        if (i >= N2 * N * Q) break;
+        const int mn0 = i % N2, r = i / N2;
+        const int n1 = r % N, q2 = r / N;
+        for (int c = 0; c < count; ++c) {
+          int j, a;
+          comb(c, j, a);
+          const T* fg1 = FG + ((j == 1 ? 2 : 0) + (a == 2 ? 1 : 0)) * Q * N2;
+          const T* t1 = T1 + (c * Q * Q + Q * q2) * N2 + mn0;
           T acc[N];
 #pragma unroll
           for (int m1 = 0; m1 < N; ++m1) acc[m1] = (T)0;
 #pragma unroll
           for (int q1 = 0; q1 < Q; ++q1) {
-            const T tv = T1[mn0 * Q * Q + q1 + Q * q2];
+            const T tv = t1[q1 * N2];
             const T* fr = fg1 + q1 * N2 + N * n1;
 #pragma unroll
             for (int m1 = 0; m1 < N; ++m1) acc[m1] += fr[m1] * tv;
           }
 #pragma unroll
-          for (int m1 = 0; m1 < N; ++m1) T2[(mn0 * N2 + m1 + N * n1) * Q + q2] += acc[m1];
+          for (int m1 = 0; m1 < N; ++m1) sum[it][m1] += acc[m1];
         }
-        __syncthreads();
       }
-      // contract q2 into X[n][m], a thread per (m0, m1, n0, n1, n2) (m0, m1
-      // fastest: neighbouring threads touch neighbouring rows of X), m2 in
-      // registers
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const int i = threadIdx.x + 256 * it;
+        if (i >= N2 * N * Q) break;
+        const int mn0 = i % N2, r = i / N2;
+        const int n1 = r % N, q2 = r / N;
+#pragma unroll
+        for (int m1 = 0; m1 < N; ++m1) T2[q2 * T2Q + n1 * T2N + m1 * N2 + mn0] = sum[it][m1];
+      }
+      __syncthreads();
+      // contract q2 into X[n][m], a thread per (mn0, m1, n1, n2), m2 in registers
+      // (the next type's T2 is written after at least one more barrier)
       const T* fg2 = FG + type * Q * N2;
       for (int i = threadIdx.x; i < N2 * N2 * N; i += blockDim.x) {
-        const int m0 = i % N, m1 = (i / N) % N, n0 = (i / N2) % N, n1 = (i / (N2 * N)) % N;
-        const int n2 = i / (N2 * N2);
-        const int mn0 = m0 + N * n0, mn1 = m1 + N * n1;
-        const T* t2 = T2 + (mn0 * N2 + mn1) * Q;
+        const int mn0 = i % N2, m1 = (i / N2) % N, n1 = (i / (N2 * N)) % N, n2 = i / (N2 * N2);
+        const int m0 = mn0 % N, n0 = mn0 / N;
+        const T* t2 = T2 + n1 * T2N + m1 * N2 + mn0;
         T acc[N];
 #pragma unroll
         for (int m2 = 0; m2 < N; ++m2) acc[m2] = (T)0;
 #pragma unroll
         for (int q2 = 0; q2 < Q; ++q2) {
-          const T tv = t2[q2];
+          const T tv = t2[q2 * T2Q];
           const T* fr = fg2 + q2 * N2 + N * n2;
 #pragma unroll
           for (int m2 = 0; m2 < N; ++m2) acc[m2] += fr[m2] * tv;
         }
         const int n = n0 + N * (n1 + N * n2);
 #pragma unroll
-        for (int m2 = 0; m2 < N; ++m2) X[n * NM + m0 + N * (m1 + N * m2)] += acc[m2];
+        for (int m2 = 0; m2 < N; ++m2) X[n * XS + m0 + N * (m1 + N * m2)] += acc[m2];
       }
-      __syncthreads();
     }
   } else {
     for (int ja = 0; ja < JA; ++ja) {
@@ -605,44 +697,54 @@ __global__ void __launch_bounds__(256) brj_block_kernel(
     }
   }
   __syncthreads();
-  // own-side trace term, face by face (face-slice modes only)
-  for (int lf = 0; lf < 2 * DIM; ++lf) {
-    const int r = lf >> 1;
-    const int vert = (lf & 1) ? P : 0;
-    const T* jd = Jd + (((long long)e * 2 * DIM + lf) * NF) * NV * NV + k * NV + l;
-    T* sJ = T1;  // [NF] face values, then [N2][Q] partial contraction
-    T* S1 = T1 + NF;
-    for (int p = threadIdx.x; p < NF; p += blockDim.x) sJ[p] = jd[(long long)p * NV * NV];
+  // own-side trace term (face-slice modes only); 3-D: every face's Jacobians and
+  // first contraction together, then face by face into X
+  if constexpr (DIM == 3) {
+    constexpr int NFC = 2 * DIM;
+    static_assert(NFC * NF <= T1SZ && NFC * N2 * Q <= T2SZ, "trace scratch");
+    T* sJ = T1;   // [NFC][NF]
+    T* S1 = T2;   // [NFC][Q p1][N2]
+    const T* FG = Y;  // products b(p, a) b(p, b) of the first type
+    const T* jd = Jd + (long long)e * NFC * NF * NV * NV + k * NV + l;
+    for (int i = threadIdx.x; i < NFC * NF; i += blockDim.x) sJ[i] = jd[(long long)i * NV * NV];
     __syncthreads();
-    if constexpr (DIM == 3) {
+    for (int i = threadIdx.x; i < NFC * N2 * Q; i += blockDim.x) {
+      const int ab = i % N2, p1 = (i / N2) % Q, lf = i / (N2 * Q);
+      T acc = (T)0;
+#pragma unroll
+      for (int p0 = 0; p0 < Q; ++p0) acc += FG[p0 * N2 + ab] * sJ[lf * NF + p0 + Q * p1];
+      S1[i] = acc;
+    }
+    __syncthreads();
+    for (int lf = 0; lf < NFC; ++lf) {
+      const int r = lf >> 1, vert = (lf & 1) ? P : 0;
       const int t0 = r == 0 ? 1 : 0, t1 = r == 2 ? 1 : 2;
-      // S1[(a0 + N b0)][p1] = sum_p0 b(p0, a0) b(p0, b0) J(p0 + Q p1)
-      for (int i = threadIdx.x; i < N2 * Q; i += blockDim.x) {
-        const int ab = i / Q, p1 = i % Q;
-        const int a0 = ab % N, b0 = ab / N;
-        T acc = (T)0;
-#pragma unroll
-        for (int p0 = 0; p0 < Q; ++p0) acc += sB1[p0 * N + a0] * sB1[p0 * N + b0] * sJ[p0 + Q * p1];
-        S1[i] = acc;
-      }
-      __syncthreads();
       for (int i = threadIdx.x; i < N2 * N2; i += blockDim.x) {
-        const int a0 = i % N, b0 = (i / N) % N, a1 = (i / N2) % N, b1 = i / (N2 * N);
+        const int ab0 = i % N2, ab1 = i / N2;
         T acc = (T)0;
 #pragma unroll
-        for (int p1 = 0; p1 < Q; ++p1)
-          acc += sB1[p1 * N + a1] * sB1[p1 * N + b1] * S1[(a0 + N * b0) * Q + p1];
+        for (int p1 = 0; p1 < Q; ++p1) acc += FG[p1 * N2 + ab1] * S1[(lf * Q + p1) * N2 + ab0];
         int mc[3], nc[3];
         mc[r] = vert;
         nc[r] = vert;
-        mc[t0] = a0;
-        mc[t1] = a1;
-        nc[t0] = b0;
-        nc[t1] = b1;
+        mc[t0] = ab0 % N;
+        mc[t1] = ab1 % N;
+        nc[t0] = ab0 / N;
+        nc[t1] = ab1 / N;
         const int m = mc[0] + N * (mc[1] + N * mc[2]), n = nc[0] + N * (nc[1] + N * nc[2]);
-        X[n * NM + m] += acc;
+        X[n * XS + m] += acc;
       }
-    } else {
+      __syncthreads();
+    }
+  }
+  for (int lf = 0; lf < (DIM == 3 ? 0 : 2 * DIM); ++lf) {
+    const int r = lf >> 1;
+    const int vert = (lf & 1) ? P : 0;
+    const T* jd = Jd + (((long long)e * 2 * DIM + lf) * NF) * NV * NV + k * NV + l;
+    T* sJ = T1;  // [NF] face values
+    for (int p = threadIdx.x; p < NF; p += blockDim.x) sJ[p] = jd[(long long)p * NV * NV];
+    __syncthreads();
+    if constexpr (DIM == 2) {
       const int t0 = 1 - r;
       for (int i = threadIdx.x; i < N2; i += blockDim.x) {
         const int a0 = i % N, b0 = i / N;
@@ -670,14 +772,14 @@ __global__ void __launch_bounds__(256) brj_block_kernel(
     for (int i = threadIdx.x; i < NM * NM; i += blockDim.x) {
       const int col = i / NM, m = i % NM;
       T a = (T)0;
-      for (int kk = 0; kk < NM; ++kk) a += sMd[kk * NM + m] * src[col * NM + kk];
-      dst[i] = a;
+      for (int kk = 0; kk < NM; ++kk) a += sMd[kk * NM + m] * src[col * XS + kk];
+      dst[col * XS + m] = a;
     }
     __syncthreads();
     T* out = blocks + (long long)e * (NV * NM) * ld;
     for (int i = threadIdx.x; i < NM * NM; i += blockDim.x) {
       const int m = i / NM, n = i % NM;
-      double val = -dta * (double)dst[n * NM + m];
+      double val = -dta * (double)dst[n * XS + m];
       if (k == l && m == n) val += 1.0;
       out[(long long)(l * NM + n) * ld + k * NM + m] = (T)val;
     }
@@ -692,11 +794,18 @@ __global__ void __launch_bounds__(256) brj_block_kernel(
       mode_coords<DIM, N>(m, mc);
       const int str = ax == 0 ? 1 : (ax == 1 ? N : N * N);
       const int base = m - mc[ax] * str;
-      double s = 0.0;
+      const T* x = src + col * XS + base;
+      T val;
+      bool done = false;
+      if constexpr (std::is_same<T, float>::value) {
+        PairSum ps;
 #pragma unroll
-      for (int kk = 0; kk < N; ++kk)
-        s += sMi[mc[ax] * N + kk] * (double)src[col * NM + base + kk * str];
-      dst[i] = (T)s;
+        for (int kk = 0; kk < N; ++kk) ps.add(sMh[mc[ax] * N + kk], sMl[mc[ax] * N + kk], x[kk * str]);
+        val = ps.value();
+        done = !ps.near(val);
+      }
+      if (!done) val = fp64_row<N>(sMi + mc[ax] * N, x, str);
+      dst[col * XS + m] = val;
     }
     __syncthreads();
     T* tmp = src;
@@ -705,13 +814,25 @@ __global__ void __launch_bounds__(256) brj_block_kernel(
   }
   // D = I - dt_a M^-1 X into rows k*NM + m, columns l*NM + n
   T* out = blocks + (long long)e * (NV * NM) * ld;
+  const double sc = -dta * idet;
+  const float sh = (float)sc, sl = (float)(sc - (double)sh);
   for (int i = threadIdx.x; i < NM * NM; i += blockDim.x) {
-    const int m = i / NM, n = i % NM;
-    double val = -dta * idet * (double)src[n * NM + m];
-    if (k == l && m == n) val += 1.0;
+    const int n = i / NM, m = i % NM;
+    const T x = src[n * XS + m];
+    T v;
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+      if (!(k == l && m == n)) {
+        PairSum ps;
+        ps.add(sh, sl, x);
+        v = ps.value();
+        done = !ps.near(v);
+      }
+    }
+    if (!done) v = fp64_scaled(sc, x, k == l && m == n ? 1.0 : 0.0);
     // stored transposed: the inverse of the transpose is the transpose of the
     // inverse, which the column-streaming block GEMV reads
-    out[(long long)(l * NM + n) * ld + k * NM + m] = (T)val;
+    out[(long long)(l * NM + n) * ld + k * NM + m] = v;
   }
 }
 
@@ -1170,9 +1291,10 @@ struct BRJImpl {
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm));
     // general elements stage the dense M^-1 beside the weights
     const int wsz = NQ * DIM * (DIM + 1);
-    constexpr int N2 = C::N * C::N;
-    constexpr int TSZ = DIM == 3 ? N2 * Q * Q + N2 * N2 * Q : 4 * N2 * Q;
-    const size_t bsm = sizeof(T) * (2 * NM * NM + (CV && NM * NM > wsz ? NM * NM : wsz) + TSZ);
+    using BS = BlockSmem<DIM, P, Q>;
+    constexpr int TSZ = BS::T1SZ + BS::T2SZ;
+    const int scratch = wsz + TSZ;
+    const size_t bsm = sizeof(T) * (2 * NM * BS::XS + (CV && NM * NM > scratch ? NM * NM : scratch));
     DG_CUDA(cudaFuncSetAttribute(brj_block_kernel<DIM, P, Q, T, CV>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm));
     const int CH = pc->wchunk;
