@@ -155,8 +155,9 @@ dg_status dg_mesh_info(dg_mesh_t m, dg_mesh_info_t* info);
 
 /* Autotuning of the sum-factorisation kernels (no counterpart in the paper,
  * whose kernels ran on CPUs): dg_autotune times every launch shape (elements
- * per CTA, threads per CTA) of the volume and lift kernels that fits one CTA's
- * shared memory, reps launches each, on the projected analytic field, and keeps
+ * per CTA, threads per CTA) of the volume kernel (vol_*, which carries the
+ * lift) and of the face kernel (lift_*: the faces of that many elements, dim
+ * each, per CTA) that fits one CTA's shared memory, reps launches each, on the projected analytic field, and keeps
  * the fastest for this mesh; result receives the choice and its times (ms per
  * launch; *_default: the shape in effect before the call, the built-in one on
  * a fresh mesh, timed also when it is not a candidate).  dg_set_tune applies a shape taken
@@ -417,7 +418,9 @@ long long dg_kernel_launches(void);
  * the library brackets each of its kernel launches with CUDA events on the
  * launch stream.  dg_profile_read synchronises the device and returns, per
  * kernel family, the launch count and summed device time since the previous
- * read (at most cap entries in out, *n set to the number written). */
+ * read (at most cap entries in out, *n set to the number written); dg_lift
+ * counts the passes of the lift, which run inside the dg_vol kernel and take
+ * their time there. */
 typedef struct {
   char name[24];
   long long launches;

@@ -1,19 +1,13 @@
-// DG residual R(u) = M^-1 L(u, t) of Sec. 3.1 (Eq. matrix-form-equations) in
-// three FP64 kernels, each in two geometry variants: axis-aligned affine
-// quads/hexes (diagonal metric, tensor-product inverse mass) and general
-// elements (curved or rotated: per-point metrics, dense inverse mass):
-//   vol_kernel   sum-factorised BwdTrans (B), collocation derivatives on the
-//                Gauss grid (D_j), fused Euler + viscous volume flux H_j
-//                weighted by w|J| and the reference metric, and the face
-//                traces of Q and grad Q (interpolation J to the faces);
-//   face_kernel  one thread per face point: Riemann flux (Roe/HLLC), the
-//                interior-penalty viscous flux and the symmetric flux S_i;
-//   lift_kernel  spreads the face fluxes back onto the Gauss grid (J^T),
-//                applies sum_j D_j^T, B^T and the inverse mass matrix
-//                |J|^-1 (M1^-1)^(x)d, adds the forcing and (for the
-//                Jacobian-free product) the finite-difference combination.
-// FP64 throughout: on GB300 this path is bound by the FP64 pipe, so every
-// stage is written to issue as few FP64 instructions as possible.
+// DG residual R(u) = M^-1 L(u, t) of Sec. 3.1 (Eq. matrix-form-equations): the
+// dispatch over (dim, P, Q) and geometry, launch shapes and their autotuning,
+// the shock sensor, the L2 projection, and the FP64 traces that the
+// preconditioner build differentiates.  The residual's own kernels are two per
+// geometry kind (axis-aligned: dg_affine.cuh; general: dg_general.cuh): faces
+// (traces, Riemann, interior-penalty and symmetric fluxes) and volume
+// (BwdTrans, derivatives, fluxes, the lift of both, M^-1, and for the
+// Jacobian-free product the finite-difference combination).  Their
+// contractions run in 64-bit fixed point on the integer pipe (dg_fix.cuh),
+// FP64 is left with the pointwise fluxes.
 #include <cstdio>
 #include <vector>
 #include "dg_internal.h"
@@ -123,7 +117,10 @@ __global__ void __launch_bounds__(32 * SENSOR_WARPS) sensor_kernel(
   sensor_element<DIM, P, Q, CV>(st, ph, geo, gg, e, sA[w], sC[w], lane, avf);
 }
 
-// ---------------------------------------------------------------- kernel 1
+// ---------------------------------------------------------------- FP64 traces
+// Traces of Q and grad Q on every element's faces, [E][2 DIM][(1+DIM) NV][NF]:
+// sum-factorised BwdTrans, collocation derivatives on the Gauss grid and
+// Lagrange extrapolation along the normal, all in FP64.
 template <int DIM, int P, int Q, bool CV>
 __global__ void __launch_bounds__(256) trace_kernel(const __grid_constant__ Tables tab,
                                                     const ElemGeo* __restrict__ geo,
