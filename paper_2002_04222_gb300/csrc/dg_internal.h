@@ -138,7 +138,6 @@ struct dg_mesh_s {
   double* hhost = nullptr;      // pinned host mirror
   // SDIRK workspace
   double* stage = nullptr;      // [DG_MAX_STAGES + 7][ndof]: E^0..E^5, S, U, R, N, U2, R2, N2
-  std::vector<std::vector<int>> elem_faces;  // host: face id of (e, lf)
   // graph replay of GMRES Arnoldi steps (one instantiated graph per step index
   // and operand set; see gmres_impl)
   struct ArnoldiGraph {
