@@ -42,8 +42,10 @@ __device__ __forceinline__ i64 mul_wide(int a, int b) {
 // largest error of the residual
 constexpr i64 FIX_HALF = 1ll << 29;
 
-// x / 2^sh to the nearest
-__device__ __forceinline__ i64 fix_shift(i64 x, int sh) {
+// x / 2^sh to the nearest, for any sh >= 0 and |x| < 2^61: from 62 on that is 0
+// (and 2^63, twice the half unit to add at 63, is not an i64)
+__host__ __device__ __forceinline__ i64 fix_shift(i64 x, int sh) {
+  sh = sh < 62 ? sh : 62;
   return (x + ((1ll << sh) >> 1)) >> sh;
 }
 

@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(256, 2) vol_gen_kernel(
     for (int vv = 0; vv < NV; ++vv) {
       int b0, bad, xh[DIM], xl[DIM];
       const int eh = fix_emax(sH[eb * NV + vv], b0);
-      const int sh = min(g_exp(eb * NV + vv, bad) - (eh + eg - 1020), 63);
+      const int sh = g_exp(eb * NV + vv, bad) - (eh + eg - 1020);
 #pragma unroll
       for (int j = 0; j < DIM; ++j) fix_split(to_fix(s1[j * ASZ + off + vv * VP], eh, 58), xh[j], xl[j]);
 #pragma unroll
