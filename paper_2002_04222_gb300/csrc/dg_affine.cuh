@@ -47,7 +47,7 @@ struct Aff {
   static constexpr int FY = imax(4 * NV * NT, DIM == 3 ? KK * NV * NF : 0);
   // shared memory in bytes of `e` elements / `f` faces per block
   static constexpr size_t vol_bytes(int e) {
-    return (size_t)e * (8 * VOL_EL + 2 * DIM * 28 + 4 * NV * 4);
+    return (size_t)e * (8 * VOL_EL + 2 * DIM * 36 + 4 * NV * 4);
   }
   static constexpr size_t face_bytes(int f) { return (size_t)f * (8 * (FX + FY) + 128 + 6 * NV * 4); }
 };
@@ -726,6 +726,7 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
     int f;           // face id
     FixScale c0, c1; // 2/h_r; (2/h_r)^2 c beta_s
   };
+  static_assert(sizeof(ElFace) <= 36, "vol_bytes");
   ElFace* ef = (ElFace*)(s1 + DIM * ASZ);       // [EPB][2 DIM]
   int* sE = (int*)(ef + EPB * 2 * DIM);         // [EPB][NV] coefficients
   int* sH = sE + EPB * NV;                      // [EPB][NV] fluxes and face data

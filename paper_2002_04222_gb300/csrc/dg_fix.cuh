@@ -16,7 +16,11 @@
 // in the inputs mark the (element, variable) bad: everything converted back
 // from it is NaN.
 #pragma once
+#include <cstring>
 #include "dg_internal.h"
+
+// (compiled for the host too, where the tests compare it with exact integers)
+#define DG_HD __host__ __device__ __forceinline__
 
 namespace dg {
 
@@ -31,10 +35,34 @@ constexpr int FIX_EBAD = 2010;  // largest exponent held; from here on (2^987) t
 // compiler sign-extends the table entries once and multiplies 64 by 64 bits;
 // from PTX multiply-adds it splits half of them into product and sum: 61
 // against 35 instructions per 36 multiply-adds.)
-__device__ __forceinline__ i64 mul_wide(int a, int b) {
+DG_HD i64 mul_wide(int a, int b) {
+#ifdef __CUDA_ARCH__
   i64 d;
   asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
   return d;
+#else
+  return (i64)a * b;
+#endif
+}
+
+// the words of a double
+DG_HD int fix_hi(double v) {
+#ifdef __CUDA_ARCH__
+  return __double2hiint(v);
+#else
+  i64 b;
+  std::memcpy(&b, &v, 8);
+  return (int)(b >> 32);
+#endif
+}
+DG_HD unsigned fix_lo(double v) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2loint(v);
+#else
+  i64 b;
+  std::memcpy(&b, &v, 8);
+  return (unsigned)b;
+#endif
 }
 
 // half a unit of a product's result, in the middle accumulator: without it
@@ -44,47 +72,51 @@ constexpr i64 FIX_HALF = 1ll << 29;
 
 // x / 2^sh to the nearest, for any sh >= 0 and |x| < 2^61: from 62 on that is 0
 // (and 2^63, twice the half unit to add at 63, is not an i64)
-__host__ __device__ __forceinline__ i64 fix_shift(i64 x, int sh) {
+DG_HD i64 fix_shift(i64 x, int sh) {
   sh = sh < 62 ? sh : 62;
   return (x + ((1ll << sh) >> 1)) >> sh;
 }
 
 // biased exponent of a double (0x7ff for infinities and NaN)
-__device__ __forceinline__ int fix_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+DG_HD int fix_exp(double v) { return (fix_hi(v) >> 20) & 0x7ff; }
 
-__device__ __forceinline__ void fix_split(i64 x, int& h, int& l) {
+DG_HD void fix_split(i64 x, int& h, int& l) {
   l = (int)x;
   h = (int)(x >> 32) + (int)((unsigned)l >> 31);  // balanced halves: x = h 2^32 + l
 }
 
 // v as an integer below 2^nb for the largest biased exponent emax >= exponent(v)
-__device__ __forceinline__ i64 to_fix(double v, int emax, int nb) {
-  const int hi = __double2hiint(v);
-  const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
-  const int d = min(emax - ((hi >> 20) & 0x7ff), 63);
+DG_HD i64 to_fix(double v, int emax, int nb) {
+  const int hi = fix_hi(v);
+  const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | fix_lo(v);
+  int d = emax - ((hi >> 20) & 0x7ff);
+  d = d < 63 ? d : 63;
   const i64 a = (i64)((m << (nb - 53)) >> d), s = (i64)(hi >> 31);
   return (a ^ s) - s;
 }
 
-// A positive or negative factor rm 2^(er - 62), 2^61 <= |rm| < 2^62 (0: rm = 0)
+// A factor of magnitude rm 2^(er - 62), 2^61 <= rm < 2^62 (0: rm = 0), its sign
+// kept apart: what is multiplied is a magnitude, cut off towards 0 on both
+// sides (a negative rm would cut its products off towards -infinity and turn
+// zeros into -1)
 struct FixScale {
   int h, l;  // balanced halves of rm
   int er;
+  int sg;    // 0 or -1
 };
-__device__ __forceinline__ FixScale fix_scale(double r) {
+DG_HD FixScale fix_scale(double r) {
   FixScale f;
-  const i64 b = __double_as_longlong(r);
-  const int E = (int)(b >> 52) & 0x7ff;
-  i64 m = ((b & 0xfffffffffffffLL) | 0x10000000000000LL) << 9;
+  const int hi = fix_hi(r), E = (hi >> 20) & 0x7ff;
+  i64 m = (i64)(((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | fix_lo(r)) << 9;
   if (E == 0) m = 0;
-  if (b < 0) m = -m;
   fix_split(m, f.h, f.l);
   f.er = E == 0 ? -4000 : E - 1022;
+  f.sg = hi >> 31;
   return f;
 }
 
 // x rm / 2^62
-__device__ __forceinline__ i64 fix_mul(i64 x, int rh, int rl) {
+DG_HD i64 fix_mul(i64 x, int rh, int rl) {
   int h, l;
   fix_split(x, h, l);
   const i64 mid = FIX_HALF + mul_wide(l, rh) + mul_wide(h, rl);
@@ -92,14 +124,15 @@ __device__ __forceinline__ i64 fix_mul(i64 x, int rh, int rl) {
 }
 
 // v r as an integer below 2^nb (nb <= 60); emax >= exponent(v) + r.er
-__device__ __forceinline__ i64 to_fix_mul(double v, const FixScale& r, int emax, int nb) {
-  const int hi = __double2hiint(v);
-  const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+DG_HD i64 to_fix_mul(double v, const FixScale& r, int emax, int nb) {
+  const int hi = fix_hi(v);
+  const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | fix_lo(v);
   const int E = (hi >> 20) & 0x7ff;
   i64 a = fix_mul((i64)(m << 7), r.h, r.l);
-  const int d = E == 0 ? 63 : min(emax - E - r.er + 60 - nb, 63);
+  int d = emax - E - r.er + 60 - nb;
+  d = E == 0 || d > 63 ? 63 : d;
   a >>= d;
-  const i64 s = (i64)(hi >> 31);
+  const i64 s = (i64)((hi >> 31) ^ r.sg);
   return (a ^ s) - s;
 }
 

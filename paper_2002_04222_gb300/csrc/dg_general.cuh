@@ -455,6 +455,7 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
         i64 m = fix_mul((i64)(((u64)(unsigned)sJ.h << 32) + (i64)sJ.l), g.cb.h, g.cb.l);
         fix_split(m, sJ.h, sJ.l);
         sJ.er += g.cb.er;
+        sJ.sg ^= g.cb.sg;
       }
 #pragma unroll
       for (int side = 0; side < 2; ++side) {

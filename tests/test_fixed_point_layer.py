@@ -33,3 +33,35 @@ def test_shift_rounds_to_the_nearest(tmp_path):
     assert len(got) == len(cases)
     for (x, sh), g in zip(cases, got):
         assert int(g) == (2 * x + (1 << sh)) // (2 << sh), (x, sh)
+
+
+def test_products_round_alike_on_both_signs(tmp_path):
+    """v r at a shared exponent, for factors of both signs (a negative
+    beta_s makes some): the magnitude is cut off towards 0 to within two units
+    of the exact product's, zeros stay 0, and the signs of v and r only change
+    the result's sign."""
+    from fractions import Fraction
+    import random
+    import struct
+    rng = random.Random(4)
+
+    def expo(v):
+        return (struct.unpack("<q", struct.pack("<d", v))[0] >> 52) & 0x7ff
+
+    vs = [0.0, 1.0, 0.75, 2.0 ** -30, 2.0 ** -70] + [rng.uniform(0.1, 1.9) * 2.0 ** -rng.randrange(8)
+                                                     for _ in range(20)]
+    rs = [1.0, 0.0, 0.3, 1.7e5, 3e-9] + [rng.uniform(0.5, 8.0) for _ in range(5)]
+    cases = [(sv * v, sr * r) for v in vs for r in rs for sv in (1, -1) for sr in (1, -1)]
+    # an exponent no product exceeds: that of v's largest plus r's
+    emax = [expo(2.0) + (expo(r) - 1022 if r else 0) for _, r in cases]
+    got = run_host(tmp_path, 'double v, r; int e; while (scanf("%la %la %d", &v, &r, &e) == 3) '
+                             'printf("%lld\\n", (long long)to_fix_mul(v, fix_scale(r), e, 58));',
+                   [f"{v.hex()} {r.hex()} {e}" for (v, r), e in zip(cases, emax)])
+    assert len(got) == len(cases)
+    by = {}
+    for (v, r), e, g in zip(cases, emax, got):
+        exact = abs(Fraction(v) * Fraction(r)) * Fraction(2) ** (58 - (e - 1022))
+        x, sign = int(g), (-1 if (v < 0) != (r < 0) else 1)
+        assert 0 <= sign * x <= exact + 1 and exact - sign * x < 3, (v, r, x)
+        by.setdefault((abs(v), abs(r)), set()).add(sign * x)
+    assert all(len(s) == 1 for s in by.values())
