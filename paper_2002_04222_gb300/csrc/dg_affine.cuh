@@ -257,7 +257,7 @@ __global__ void __maxnreg__(80) face_fix_kernel(
   double* sX = sm;                                   // [FPB][FX]
   double* sY = sX + FPB * A::FX;                     // [FPB][FY]
   FaceInfo* info = (FaceInfo*)(sY + FPB * A::FY);    // [FPB]
-  int* sE = (int*)(info + FPB);                      // [FPB][2][NV] coefficients, both sides
+  int* sE = (int*)(info + FPB);                      // [FPB][2][NV] coefficients of each side
   int* sS = sE + FPB * 2 * NV;                       // [FPB][3][NV] outputs f, T, S_n
   int* sT = sS + FPB * 3 * NV;                       // [FPB][NV] scaled tangential S
   const int f0 = blockIdx.x * FPB;
@@ -306,13 +306,19 @@ __global__ void __maxnreg__(80) face_fix_kernel(
         m = max(m, fix_exp(val));
       }
       m = __reduce_max_sync(0xffffffffu, m);
-      if (lane == 0) sE[fb * 2 * NV + sv] = m;
+      if (lane == 0) {
+        sE[fb * 2 * NV + sv] = m;
+        // (a boundary face counts its side twice)
+        if (info[fb].bc != 0) sE[fb * 2 * NV + (1 - side) * NV + vv] = m;
+      }
     }
   }
   __syncthreads();
   // face coefficients per (face, variable, tangential mode): both sides'
   // values, their sum, and the sum of the normal derivatives scaled by 2/h_n
-  // over the larger of the two (a boundary face counts its side twice)
+  // over the larger of the two.  A side's values keep its own exponent (beside
+  // a neighbour 10^8 times larger one exponent for both left them 32 bits of
+  // the 53 that a double holds); the sums take the larger of the two.
   i64* C0 = (i64*)sY;
   for (int idx = tid; idx < nf * NV * NT; idx += nth) {
     const int fb = idx / (NV * NT), rem = idx - fb * NV * NT;
@@ -323,7 +329,8 @@ __global__ void __maxnreg__(80) face_fix_kernel(
     const int s0 = r == 0 ? N : 1, s1 = r == 2 ? N : N * N;
     const int off = (DIM == 3 ? (l % N) * s0 + (l / N) * s1 : l * s0);
     int bad;
-    const int em = fix_emax(max(sE[(fb * 2) * NV + vv], sE[(fb * 2 + 1) * NV + vv]), bad);
+    const int es[2] = {fix_emax(sE[(fb * 2) * NV + vv], bad), fix_emax(sE[(fb * 2 + 1) * NV + vv], bad)};
+    const int em = max(es[0], es[1]);
     i64 val[2] = {0, 0}, der[2] = {0, 0};
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
@@ -332,13 +339,14 @@ __global__ void __maxnreg__(80) face_fix_kernel(
       int xh[N], xl[N];
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        const i64 x = to_fix(src[k * sn], em, 59);
+        const i64 x = to_fix(src[k * sn], es[side], 59);
         if (k == (side == 0 ? P : 0)) val[side] = x;
         fix_split(x, xh[k], xl[k]);
       }
       // the side below has the face at its upper end
       const i64 d = fix_dot<N>(xh, xl, ft.dp[1 - side]);
-      der[side] = side == 0 ? fix_mul(d, g.rhA[0], g.rhA[1]) : fix_mul(d, g.rhB[0], g.rhB[1]);
+      der[side] = fix_shift(
+          side == 0 ? fix_mul(d, g.rhA[0], g.rhA[1]) : fix_mul(d, g.rhB[0], g.rhB[1]), em - es[side]);
     }
     if (g.eA < 0) {
       val[0] = val[1];
@@ -352,7 +360,7 @@ __global__ void __maxnreg__(80) face_fix_kernel(
     o[VALA * NV * NT] = val[0];
     o[VALB * NV * NT] = val[1];
     o[DN * NV * NT] = der[0] + der[1];
-    o[DT * NV * NT] = val[0] + val[1];
+    o[DT * NV * NT] = fix_shift(val[0], em - es[0]) + fix_shift(val[1], em - es[1]);
   }
   __syncthreads();
   i64* C1 = (i64*)sX;  // 3-D: first tangential direction on its points, [4][NV][N][RQ]
@@ -380,8 +388,11 @@ __global__ void __maxnreg__(80) face_fix_kernel(
     const int kind = idx / (nf * NV * NL), rem = idx - kind * nf * NV * NL;
     const int fb = rem / (NV * NL), vq = rem - fb * NV * NL;
     const int vv = vq / NL, q0 = vq - vv * NL;
-    int bad;
-    int se = fix_emax(max(sE[(fb * 2) * NV + vv], sE[(fb * 2 + 1) * NV + vv]), bad) - 1022 - 59;
+    int badA, badB;
+    const int esA = fix_emax(sE[(fb * 2) * NV + vv], badA), esB = fix_emax(sE[(fb * 2 + 1) * NV + vv], badB);
+    const int em = max(esA, esB);
+    const int bad = kind == VALA ? badA : (kind == VALB ? badB : badA | badB);
+    int se = (kind == VALA ? esA : (kind == VALB ? esB : em)) - 1022 - 59;
     int xh[N], xl[N];
     const i64* src;
     bool db;
@@ -393,7 +404,8 @@ __global__ void __maxnreg__(80) face_fix_kernel(
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         i64 x = src[k * RQ];
-        if (db) x += src[k * RQ + (VALB - VALA) * NV * N * RQ];
+        if (db)
+          x = fix_shift(x, em - esA) + fix_shift(src[k * RQ + (VALB - VALA) * NV * N * RQ], em - esB);
         fix_split(x, xh[k], xl[k]);
       }
     } else {

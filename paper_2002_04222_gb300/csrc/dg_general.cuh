@@ -162,7 +162,8 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     }
   }
   __syncthreads();
-  // per side: the face's coefficients and those of the normal derivative
+  // per side, at its own exponent: the face's coefficients and those of the
+  // normal derivative
   i64* C0 = (i64*)sY;  // [2 side][2][NV][NT]
   for (int idx = tid; idx < nf * 2 * NV * NT; idx += nth) {
     const int fb = idx / (2 * NV * NT), rem = idx - fb * 2 * NV * NT;
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     const double* src = sX + fb * A::GX + sv * NM +
                         (DIM == 3 ? (l % N) * s0 + (l / N) * s1 : l * s0);
     int bad, xh[N], xl[N];
-    const int em = fix_emax(max(sE[(fb * 2) * NV + vv], sE[(fb * 2 + 1) * NV + vv]), bad);
+    const int em = fix_emax(sE[fb * 2 * NV + sv], bad);
     i64 first = 0, last = 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
@@ -212,8 +213,8 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     __syncthreads();
   }
   // last tangential direction: fields [NFLD][NV][NF], the values as doubles,
-  // the derivatives as integers of one scale: 0, 1 values; 2 + DIM side + (0
-  // normal, 1.. tangential)
+  // the derivatives as integers of one scale (both sides' too): 0, 1 values;
+  // 2 + DIM side + (0 normal, 1.. tangential)
   const int eT = max(ft.edp + ft.eB, ft.eDB) + (DIM == 3 ? ft.eB : 0);
   for (int idx = tid; idx < A::NFLD * nf * NV * NL; idx += nth) {
     const int kind = idx / (nf * NV * NL), rem = idx - kind * nf * NV * NL;
@@ -241,13 +242,15 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
       for (int q = 0; q < Q; ++q) y[q] = fix_dot<N>(xh, xl, ft.B + q * N);
     }
     double* o = (DIM == 3 ? sY + fb * A::GY : sX + fb * A::GX) + (kind * NV + vv) * NF + q0;
+    int bad;
+    const int es = fix_emax(sE[(fb * 2 + side) * NV + vv], bad);
     if (kind < 2) {
-      int bad;
-      const int se = fix_emax(max(sE[(fb * 2) * NV + vv], sE[(fb * 2 + 1) * NV + vv]), bad) - 1022 -
-                     59 + (DIM - 1) * ft.eB;
+      const int se = es - 1022 - 59 + (DIM - 1) * ft.eB;
 #pragma unroll
       for (int q = 0; q < Q; ++q) o[q * NL] = fix_to_double(y[q], se, bad);
     } else {
+      int other;
+      sh += max(fix_emax(sE[(fb * 2 + 1 - side) * NV + vv], other) - es, 0);
 #pragma unroll
       for (int q = 0; q < Q; ++q) ((i64*)o)[q * NL] = fix_shift(y[q], sh);
     }

@@ -185,3 +185,35 @@ def test_launch_shapes_give_the_same_bits(dgl, name, general):
                 tried += 1
                 assert torch.equal(m.residual(u), r), (ve, vt, lt)
     assert tried > 4
+
+
+@pytest.mark.parametrize("ratio", [1e4, 1e8])
+@pytest.mark.parametrize("shape", [(4, 2), (4, 1, 2)])
+@pytest.mark.parametrize("general", [False, True])
+def test_a_side_keeps_its_digits_beside_a_much_larger_neighbour(dgl, general, shape, ratio):
+    """Supersonic flow from light elements (i = 2, 3) into ones `ratio` times
+    denser (i = 0, 1): the upwinded flux of the face between them is the light
+    side's alone, so the weak form on the light elements beside it is as exact
+    as without the jump.  Bound: 64 times those elements' own rounding floor
+    (the parity tests'), for the general kernels plus cond(M) 2^-53."""
+    P, d = 2, len(shape)
+    c = (w.vortex_case(n=4, P=P) if d == 2 else w.small_tgv_case((4, 1, 2), P=P))
+    mesh = w.box_mesh([np.linspace(0.0, 1.0, n + 1) for n in shape], (True,) * d)
+    ph = c.phys
+    ph.viscous, ph.riemann, ph.Ma = False, 1, 1.0
+    dg = DG(mesh, P, c.Q, ph)
+    rho, vel = 1.0, np.array([-3.0, 0.1, 0.05][:d])
+    prim = np.concatenate([[rho], rho * vel, [rho / ph.gamma / (ph.gamma - 1.0) + 0.5 * rho * vel @ vel]])
+    u = prim[None, :, None] * (dg.one_coeffs()[None, None, :]
+                               + 0.02 * np.random.default_rng(2).standard_normal((dg.E, d + 2, dg.nm)))
+    i = np.arange(dg.E) % shape[0]
+    u[i < 2] *= ratio
+    sel = i == 2
+    L = dg.rhs(u)
+    s = np.sign(np.random.default_rng(0).standard_normal(u.shape))
+    tol = 64 * np.linalg.norm((dg.rhs(u * (1 + 2.0 ** -52 * s)) - L)[sel]) / np.linalg.norm(L[sel])
+    if general:
+        tol += np.linalg.cond(np.einsum("qm,eq,qn->emn", dg.B, dg.wJ, dg.B)).max() * 2.0 ** -53
+    got = weak(dg, dgl.Mesh(quadratic(mesh) if general else mesh, P, c.Q, ph).residual(dev(u)).cpu().numpy())
+    assert tol < 3e-10
+    assert rel(got[sel], L[sel]) < tol
