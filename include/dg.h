@@ -22,6 +22,7 @@
  *    (dim, P, Q) or feature the compiled library does not provide, DG_ERR_CUDA for a
  *    CUDA failure (sticky errors included), DG_ERR_OOM when device memory
  *    runs out, DG_ERR_NONFINITE when a norm is not finite,
+ *    DG_ERR_TIMEOUT when a bounded wait of a kernel ran out,
  *    DG_ERR_NOT_CONVERGED when an iteration cap is hit (stats are filled and
  *    the output holds the last iterate).
  *  - Handles are not thread-safe; one handle may be used by one host thread
@@ -249,6 +250,15 @@ dg_status dg_precond_build(dg_mesh_t m, const double* u, double t, double dt_a,
  * out must not alias q. */
 dg_status dg_precond_apply(dg_precond_t p, const double* q, double* out, void* stream);
 dg_status dg_precond_destroy(dg_precond_t p);
+/* On meshes whose elements are all resident on the GPU at once the solvers run
+ * an application as one cooperative launch whose blocks wait for one another
+ * between sweeps.  The waits are bounded: after `polls` looks at the counter
+ * (about 50 ns each; 2^22 unless set here) a block gives up, and the solve
+ * returns DG_ERR_TIMEOUT.  From then on the solvers apply p sweep by sweep;
+ * dg_precond_build takes the one launch up again.  With 0 every wait gives up
+ * (for tests of the caller's error path).  Returns the former limit, or
+ * DG_ERR_ARG. */
+int dg_precond_wait_limit(dg_precond_t p, int polls);
 
 /* Restarted right-preconditioned GMRES (Sec. 3.2; Saad & Schultz) for
  * (I - dt_a dR/du(u)) x = b with the Jacobian-free product at (u, r_u):

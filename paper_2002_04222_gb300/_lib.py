@@ -136,13 +136,17 @@ SIGNATURES = {
     "dg_profile_read": [ctypes.POINTER(KernelTime), I, ctypes.POINTER(I)],
     "dg_peak_fp64": [I, ctypes.POINTER(D), VP],
 }
+# those that return a value of their own (an int) instead of a status
+VALUES = {
+    "dg_precond_wait_limit": [VP, I],
+}
 
 
 def load(path=LIB_PATH):
     if not os.path.exists(path):
         raise ImportError(f"{path} is missing: build it with paper_2002_04222_gb300.build.build()")
     lib = ctypes.CDLL(path)
-    for name, args in SIGNATURES.items():
+    for name, args in {**SIGNATURES, **VALUES}.items():
         fn = getattr(lib, name)
         fn.argtypes = args
         fn.restype = {"dg_status_string": ctypes.c_char_p,

@@ -809,7 +809,9 @@ dg_status dg_gmres(dg_mesh_t m, dg_precond_t p, const double* u, const double* r
   if (cfg->restart < 1 || cfg->restart > MAX_RESTART || cfg->max_cycles < 1 || !(cfg->rtol > 0.0))
     return DG_ERR_ARG;
   if (p && precond_mesh(p) != m) return DG_ERR_ARG;
-  return gmres_impl(m, p, u, r_u, t, dt_a, b, x, cfg, stats, (cudaStream_t)stream);
+  return precond_failure(
+      p, gmres_impl(m, p, u, r_u, t, dt_a, b, x, cfg, stats, (cudaStream_t)stream),
+      (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------- SDIRK, BDF2
@@ -958,7 +960,7 @@ static dg_status newton_stage(dg_mesh_s* m, const dg_sdirk_cfg* cfg, dg_precond_
     }
     if (o.it >= cfg->max_newton) break;
     dg_gmres_stats gs{};
-    dg_status g = gmres_impl(m, P, U, R, ti, dta, Nn, dx, &cfg->gmres, &gs, s);
+    dg_status g = precond_failure(P, gmres_impl(m, P, U, R, ti, dta, Nn, dx, &cfg->gmres, &gs, s), s);
     if (g != DG_OK && g != DG_ERR_NOT_CONVERGED) return g;
     o.gits += gs.iters;
     DG_TRY(axpby(U, 1.0, dx, 1.0, n, s));

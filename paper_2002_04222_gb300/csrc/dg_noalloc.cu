@@ -122,7 +122,7 @@ extern "C" dg_status dg_gmres_noalloc(dg_mesh_t m, dg_precond_t p, const double*
       DG_CUDA(cudaMemcpyAsync(hh, hd, sizeof(double) * 3 * (mr + 2), cudaMemcpyDeviceToHost, s));
       DG_CUDA(cudaStreamSynchronize(s));
       const double hn = std::sqrt(hh[2 * (mr + 2)]);
-      if (!std::isfinite(hn)) return DG_ERR_NONFINITE;
+      if (!std::isfinite(hn)) return precond_failure(p, DG_ERR_NONFINITE, s);
       for (int i = 0; i <= k; ++i) H[(size_t)i * mr + k] = hh[i] + hh[(mr + 2) + i];
       H[(size_t)(k + 1) * mr + k] = hn;
       for (int i = 0; i < k; ++i) {

@@ -26,6 +26,7 @@
 #include <cuda_bf16.h>
 #include <new>
 #include <type_traits>
+#include <utility>
 #include <vector>
 #include "dg_internal.h"
 #include "dg_physics.cuh"
@@ -1493,6 +1494,22 @@ dg_status precond_solver_apply(dg_precond_s* pc, const double* q, double* out, c
   return precond_one_launch(pc) ? dispatch_coop_apply(pc, q, out, s) : precond_sweeps(pc, q, out, s);
 }
 
+static unsigned long long next_gen() {
+  static unsigned long long g_gen = 0;
+  return __atomic_add_fetch(&g_gen, 1ULL, __ATOMIC_RELAXED);
+}
+
+dg_status precond_failure(dg_precond_s* pc, dg_status st, cudaStream_t s) {
+  if (st != DG_ERR_NONFINITE || !pc || !pc->coop) return st;
+  unsigned long long mark = 0;
+  DG_CUDA(cudaMemcpyAsync(&mark, pc->bar + 1, sizeof(mark), cudaMemcpyDeviceToHost, s));
+  DG_CUDA(cudaStreamSynchronize(s));
+  if (mark == 0) return st;
+  pc->coop = 0;
+  pc->gen = next_gen();  // graphs that captured the one launch are not replayed
+  return DG_ERR_TIMEOUT;
+}
+
 static constexpr size_t kMaxGraphs = 128;
 
 void precond_drop_graphs(dg_precond_s* pc) {
@@ -1673,21 +1690,23 @@ dg_status dg_precond_build(dg_mesh_t m, const double* u, double t, double dt_a,
   }
   // the captured sweeps hold J, omega and the launch shapes: a rebuild re-captures
   precond_drop_graphs(p);
-  static unsigned long long g_gen = 0;
   // (the sweeps take J, omega, dt_a and their form by value; everything else by pointer
   // into buffers that a rebuild refills in place)
   if (p->gen == 0 || p->J != cfg->J || p->omega != cfg->omega || p->dt_a != dt_a ||
-      p->fused != (cfg->fused != 0))
-    p->gen = __atomic_add_fetch(&g_gen, 1ULL, __ATOMIC_RELAXED);
+      p->fused != (cfg->fused != 0) || p->coop != p->coop_fits)
+    p->gen = next_gen();
+  p->coop = 0;  // (until its buffers are there)
   if (!p->bar && !full) {
-    p->coop = dispatch_coop_apply(p, nullptr, nullptr, s) == DG_OK;
     DG_CUDA(cudaMalloc((void**)&p->bar, 2 * sizeof(unsigned long long)));
-    DG_CUDA(cudaMemset(p->bar, 0, 2 * sizeof(unsigned long long)));
+    p->coop_fits = dispatch_coop_apply(p, nullptr, nullptr, s) == DG_OK;
   }
-  if ((cfg->fused || p->coop) && !p->qh2) {
+  if ((cfg->fused || p->coop_fits) && !p->qh2) {
     DG_CUDA(cudaMalloc((void**)&p->qh2, sizeof(double) * (size_t)m->ndof));
-    DG_CUDA(cudaMemset(p->qh2, 0, sizeof(double) * (size_t)m->ndof));
+    DG_CUDA(cudaMemsetAsync(p->qh2, 0, sizeof(double) * (size_t)m->ndof, s));
   }
+  // a rebuild clears the failure mark and takes the one launch up again
+  if (p->coop_fits) DG_CUDA(cudaMemsetAsync(p->bar, 0, 2 * sizeof(unsigned long long), s));
+  p->coop = p->coop_fits;
   p->fused = cfg->fused != 0;
   p->use_graphs = cfg->graphs;
   p->tc_invert = cfg->tc_invert;
@@ -1700,6 +1719,12 @@ dg_status dg_precond_build(dg_mesh_t m, const double* u, double t, double dt_a,
 dg_status dg_precond_apply(dg_precond_t p, const double* q, double* out, void* stream) {
   if (!p || !q || !out || q == out) return DG_ERR_ARG;
   return precond_apply_impl(p, q, out, (cudaStream_t)stream);
+}
+
+int dg_precond_wait_limit(dg_precond_t p, int polls) {
+  if (!p || polls < 0) return DG_ERR_ARG;
+  if (p->wait_polls != polls) p->gen = next_gen();  // captured launches hold the limit
+  return std::exchange(p->wait_polls, polls);
 }
 
 dg_status dg_precond_destroy(dg_precond_t p) {

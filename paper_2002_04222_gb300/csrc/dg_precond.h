@@ -34,8 +34,10 @@ struct dg_precond_s {
   int fused = 0;          // sweeps j >= 2 as one off-diagonal + block kernel
   double* qh2 = nullptr;  // [ndof] second iterate buffer of the fused sweeps and of the
                           // one-launch apply (lazily allocated)
-  int coop = 0;           // every element resident at once: the solvers apply in one launch
+  int coop_fits = 0;      // every element resident at once: one launch can apply
+  int coop = 0;           // the solvers may apply in one launch (off after a wait that ran out)
   unsigned long long* bar = nullptr;  // [2] its counter and its failure mark
+  int wait_polls = 1 << 22;           // its waits' limit
   // terms 4-5 of the element Jacobian (full_jacobian): per element face and
   // point, K = s wJ dH/d grad Q [k][j][l], S_own / S_nbr = c wJ dS/dQ [i][k][l]
   int full = 0;
@@ -59,6 +61,10 @@ dg_status precond_sweeps(dg_precond_s* p, const double* q, double* out, cudaStre
 dg_status dispatch_coop_apply(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
 bool precond_one_launch(const dg_precond_s* p);
 dg_status precond_solver_apply(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
+// the status of a solve with p that ended in st: a non-finite value that a wait
+// of the one-launch apply left is DG_ERR_TIMEOUT, and p is applied by the
+// separate sweeps from then on
+dg_status precond_failure(dg_precond_s* p, dg_status st, cudaStream_t s);
 void precond_drop_graphs(dg_precond_s* p);
 // in-place inversion of E blocks nb x nb (row stride ld), panel in registers
 // (dg_invert.cu); supported for nb up to 640 (FP32) / 384 (FP64)

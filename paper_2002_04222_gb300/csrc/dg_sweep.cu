@@ -74,17 +74,17 @@ static dg_status sweep_launch(dg_precond_s* pc, const double* qprev, const doubl
 // for bit.  Between sweeps the blocks meet at a counter in global memory
 // (bar[0], only ever increased; J and the grid may change between launches
 // because every launch leaves it at a multiple of its own grid); the wait is
-// bounded, and a block that gives up marks bar[1] and leaves NaN, as does
-// every later launch.
-constexpr int COOP_SPINS = 1 << 22;
-__device__ __forceinline__ bool grid_meet(unsigned long long* bar) {
+// bounded (`polls`, some 50 ns each), and a block that gives up marks bar[1]
+// and leaves NaN, as does every later launch until a solver reads the mark
+// (precond_failure) or a rebuild clears it.
+__device__ __forceinline__ bool grid_meet(unsigned long long* bar, int polls) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned long long g = gridDim.x, old = atomicAdd(bar, 1ULL);
     const unsigned long long want = (old / g + 1) * g;
-    int left = COOP_SPINS;
+    int left = polls;
     while (*(volatile unsigned long long*)bar < want && left > 0) {
       --left;
       __nanosleep(32);
@@ -103,7 +103,7 @@ __global__ void DG_DIAG_BOUNDS(TB)
                           const double* __restrict__ minv, const TJ* __restrict__ Jo,
                           const int32_t* __restrict__ nbr, const double* __restrict__ q, double dta,
                           const TB* __restrict__ blocks, int nb, int ld, int split, double omega,
-                          int J, double* qa, double* qb, double* out, unsigned long long* bar) {
+                          int J, double* qa, double* qb, double* out, unsigned long long* bar, int polls) {
   using TA = typename Vec16<TB>::TA;
   constexpr int NTH = sizeof(TB) == 2 ? 512 : 256;
   extern __shared__ unsigned char smraw[];
@@ -118,7 +118,7 @@ __global__ void DG_DIAG_BOUNDS(TB)
   if (omega != 1.0)  // (the thread that wrote an entry scales it)
     for (int r = threadIdx.x; r < nb; r += blockDim.x) cur[(long long)e * nb + r] *= omega;
   for (int j = 1; j < J; ++j) {
-    ok = grid_meet(bar) && ok;
+    ok = grid_meet(bar, polls) && ok;
     double* nxt = j == J - 1 ? out : (cur == qa ? qb : qa);
     offdiag_element<DIM, P, Q, TA, TJ, CV, NTH, true>(
         tab, geo, minv, Jo, nbr, cur, q, dta, e, [&](int i, double v) { sy[i] = (TA)v; });
@@ -165,7 +165,7 @@ static dg_status coop_launch(dg_precond_s* pc, const double* q, double* out, cud
   DG_CUDA(cudaLaunchKernelEx(&c, kernel, m->tab, (const ElemGeo*)m->geo, (const double*)m->minv,
                              (const TJ*)pc->jo, (const int32_t*)pc->nbr, q, pc->dt_a,
                              (const TB*)pc->blocks, nb, ld, split, pc->omega, pc->J, pc->qh, pc->qh2,
-                             out, pc->bar));
+                             out, pc->bar, pc->wait_polls));
   DG_LAUNCHED(1);
   return DG_OK;
 }
