@@ -630,7 +630,7 @@ static dg_status arnoldi_step_ops(dg_mesh_s* m, dg_precond_s* p, const double* u
   const double* zk = vk;
   if (p) {
     double* zz = V + (size_t)(mr + 1) * n + (size_t)k * n;
-    DG_TRY(precond_solver_apply(p, vk, zz, s));
+    DG_TRY(precond_solver_apply(p, vk, zz, true, s));
     zk = zz;
   }
   double* w = V + (size_t)(k + 1) * n;
@@ -747,10 +747,10 @@ static dg_status gmres_impl(dg_mesh_s* m, dg_precond_s* p, const double* u, cons
         const double* zk = vk;
         if (p) {
           double* zz = Z + (size_t)k * n;
-          if (precond_one_launch(p))
-            DG_TRY(precond_solver_apply(p, vk, zz, s));
-          else
+          if (p->use_graphs && !profiling_on())
             DG_TRY(precond_apply_impl(p, vk, zz, s));
+          else
+            DG_TRY(precond_solver_apply(p, vk, zz, false, s));
           zk = zz;
         }
         DG_TRY(apply_A(m, u, r_u, t, dta, zk, w, s));

@@ -112,7 +112,7 @@ extern "C" dg_status dg_gmres_noalloc(dg_mesh_t m, dg_precond_t p, const double*
         double* zz = Z + (size_t)k * n;
         // launches, never the graph replay: capturing and instantiating a graph
         // allocates (this is what the replay of dg_gmres runs)
-        DG_TRY(precond_solver_apply(p, vk, zz, s));
+        DG_TRY(precond_solver_apply(p, vk, zz, false, s));
         zk = zz;
       }
       double* w = V + (size_t)(k + 1) * n;

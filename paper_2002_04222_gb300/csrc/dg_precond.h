@@ -56,11 +56,13 @@ dg_status dispatch_sweep(dg_precond_s* p, const double* qprev, const double* q, 
                          cudaStream_t s);
 // the apply as plain kernel launches on s (for capture inside a larger graph)
 dg_status precond_sweeps(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
-// the apply of the solvers: one cooperative launch where the elements fit the
-// GPU together (dg_sweep.cu; out = nullptr asks whether they do), else the above
+// the apply of the solvers (captured: inside a graph): where the elements fit
+// the GPU together (dg_sweep.cu; out = nullptr asks whether they do) one
+// cooperative launch or the fused sweeps, else the above
 dg_status dispatch_coop_apply(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
 bool precond_one_launch(const dg_precond_s* p);
-dg_status precond_solver_apply(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
+dg_status precond_solver_apply(dg_precond_s* p, const double* q, double* out, bool captured,
+                               cudaStream_t s);
 // the status of a solve with p that ended in st: a non-finite value that a wait
 // of the one-launch apply left is DG_ERR_TIMEOUT, and p is applied by the
 // separate sweeps from then on
