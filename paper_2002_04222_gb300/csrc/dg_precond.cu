@@ -1488,34 +1488,39 @@ dg_status precond_sweeps(dg_precond_s* pc, const double* q, double* out, cudaStr
   return DG_OK;
 }
 
-// The solvers' application on meshes whose elements are all resident at once.
-// Measured on 8 to 900 elements, 2-D P = 1..6 and 3-D P = 1..4, every
-// precision (us per BRJ(7), one launch / the handle's own sweeps):
-//  - replayed from a graph the sweeps' launches follow without gaps, and the
-//    fused ones win (one launch of them prefetches its block, the cooperative
-//    one does not): 3-D P = 3 FP32 E = 216 245 / 217, 2-D P = 2 FP32 E = 64
-//    35 / 32, BF16 P = 1 57 / 41.  So a captured application is the fused sweeps.
-//  - launched one by one the two-kernel sweeps pay 2J-1 gaps: one launch wins
-//    (2-D P = 2 FP64 E = 64 43 / 66, E = 900 86 / 112; 3-D P = 2 FP32 E = 64 73 / 105)
-//    until a block takes longer than its gap: 3-D P = 3, curved, FP32 E = 800
-//    547 / 526, fused 514.  From 320 unknowns an element on, the fused sweeps.
-//  - the fused sweeps have half the gaps: against them one launch wins up to
+// The solvers' application on meshes whose elements are all resident at once:
+// one launch or the fused sweeps, the same bits.  Measured on 8 to 900 elements,
+// 2-D P = 1..6 and 3-D P = 1..4, every precision (us per BRJ(7), one launch /
+// the handle's own sweeps).
+//  - Launched one by one, the two-kernel sweeps pay 2J-1 gaps: one launch wins
+//    (2-D P = 2 FP64 E = 64 43 / 66, E = 900 86 / 112; 3-D P = 2 FP32 E = 64
+//    73 / 105) until a block takes longer than its gap: 3-D P = 3, curved, FP32
+//    E = 800 547 / 526, fused 514.  From 320 unknowns an element on, never.
+//  - The fused sweeps have half the gaps: against them one launch wins up to
 //    100 unknowns an element (2-D P = 2 FP64 E = 64 44 / 54, P = 4 FP32 E = 900
-//    81 / 82; not BF16 blocks of 16 unknowns: 60 / 56), up to 196 while an SM
+//    81 / 82; not BF16 blocks of 16 unknowns: 60 / 56), beyond that while an SM
 //    has one block (3-D P = 2 FP32 E = 64 73 / 80, E = 343 101 / 95; 2-D P = 6
 //    FP32 E = 64 74 / 82, E = 900 208 / 185).
-// Every form gives the same bits.  Per-kernel profiling keeps the sweeps apart.
-bool precond_one_launch(const dg_precond_s* pc) {
-  if (!pc->coop || profiling_on()) return false;
-  if (!pc->fused) return pc->nb < 320;
-  if (pc->precision == DG_PREC_BF16 && pc->nb < 32) return false;
-  return pc->nb <= 100 || (pc->nb < 320 && pc->mesh->E <= 152);
+//  - Replayed from a graph the launches have no gaps, and the fused sweeps win
+//    (each prefetches its block, the one launch does not): 3-D P = 3 FP32 E = 216
+//    245 / 217, 2-D P = 2 FP32 E = 64 35 / 32.  Against the two-kernel sweeps one
+//    launch wins (2-D P = 2 FP64 E = 64 42 / 45, 3-D P = 2 FP32 71 / 83) but for
+//    BF16 blocks of 16 unknowns (57 / 47) and more than three blocks an SM (3-D
+//    P = 1 FP32 E = 512 54 / 51, E = 729 60 / 54; FP64 blocks still: E = 900 2-D
+//    P = 2 85 / 84, P = 4 240 / 260).
+// Per-kernel profiling keeps the handle's own sweeps.
+static bool precond_one_launch(const dg_precond_s* pc, bool captured) {
+  if (pc->nb >= 320) return false;
+  const bool small_bf16 = pc->precision == DG_PREC_BF16 && pc->nb < 32;
+  const int E = pc->mesh->E;
+  if (pc->fused) return !captured && !small_bf16 && (pc->nb <= 100 || E <= 152);
+  return !captured || (!small_bf16 && (pc->precision == DG_PREC_FP64 || E <= 3 * 152));
 }
 dg_status precond_solver_apply(dg_precond_s* pc, const double* q, double* out, bool captured,
                                cudaStream_t s) {
-  if (!captured && precond_one_launch(pc)) return dispatch_coop_apply(pc, q, out, s);
-  if (pc->coop && !profiling_on()) return precond_sweeps_fused(pc, q, out, s);
-  return precond_sweeps(pc, q, out, s);
+  if (!pc->coop || profiling_on()) return precond_sweeps(pc, q, out, s);
+  if (precond_one_launch(pc, captured)) return dispatch_coop_apply(pc, q, out, s);
+  return precond_sweeps_fused(pc, q, out, s);
 }
 
 static unsigned long long next_gen() {

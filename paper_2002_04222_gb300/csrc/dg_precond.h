@@ -60,7 +60,6 @@ dg_status precond_sweeps(dg_precond_s* p, const double* q, double* out, cudaStre
 // the GPU together (dg_sweep.cu; out = nullptr asks whether they do) one
 // cooperative launch or the fused sweeps, else the above
 dg_status dispatch_coop_apply(dg_precond_s* p, const double* q, double* out, cudaStream_t s);
-bool precond_one_launch(const dg_precond_s* p);
 dg_status precond_solver_apply(dg_precond_s* p, const double* q, double* out, bool captured,
                                cudaStream_t s);
 // the status of a solve with p that ended in st: a non-finite value that a wait
