@@ -47,7 +47,7 @@ struct Aff {
   static constexpr int FY = imax(4 * NV * NT, DIM == 3 ? KK * NV * NF : 0);
   // shared memory in bytes of `e` elements / `f` faces per block
   static constexpr size_t vol_bytes(int e) {
-    return (size_t)e * (8 * VOL_EL + 2 * DIM * 36 + 4 * NV * 4);
+    return (size_t)e * (8 * VOL_EL + 2 * DIM * 32 + 4 * NV * 4);
   }
   static constexpr size_t face_bytes(int f) { return (size_t)f * (8 * (FX + FY) + 128 + 6 * NV * 4); }
 };
@@ -233,9 +233,58 @@ struct FaceInfo {
   double hn, ht[2];  // half of the largest 2/h_n, halves of the tangential 2/h_t
   int rhA[2], rhB[2];  // 2/h_n of each side over the largest, 62-bit halves
   FixScale ct[2];    // c beta_s 2/h_t
+  __device__ __forceinline__ void side(int s, int& e, int& lf) const {
+    e = s == 0 ? eA : eB;
+    lf = 2 * r + 1 - s;  // the side below has the face at its upper end
+  }
 };
 
 static_assert(sizeof(FaceInfo) <= 128, "face_bytes");
+
+// ------------------------------------------------------------ sides far apart
+// Both sides' coefficients enter the face kernel at the larger of their two
+// exponents, 59 bits: a side whose variable is more than 2^6 smaller than its
+// neighbour's has fewer than a double's 53 left (32 beside one 10^8 times
+// larger).  The sums of the derivatives need no more, but a flux can be that
+// side's alone, so its values are then evaluated again from its coefficients
+// in FP64, over those from the integers.  Out of line: blocks without such a
+// face pay for one test (an exponent a side all the way through cost the kernel
+// 1.5 to 3%, and the 8x8 P = 2 residual 2 of 27 us).
+__device__ __forceinline__ bool far_below(int e, int other) { return other - max(e, FIX_EMIN) > 6; }
+
+// the values of every smaller side, fields 0 and 1 of fld [face][stride]
+template <int DIM, int P, int Q, class Info>
+__device__ __noinline__ void own_values(const FixTab& ft, const Info* info, const int* sE, int nf,
+                                        const double* __restrict__ u, const double* __restrict__ v,
+                                        double eps, double* fld, int stride) {
+  using A = Aff<DIM, P, Q>;
+  constexpr int N = A::N, NV = A::NV, NM = A::NM, NF = A::NF;
+  auto B = [&](int q, int k) {  // psi_k(x_q)
+    const int2 c = ft.B[q * N + k];
+    return ldexp(fma((double)c.x, 4294967296.0, (double)c.y), ft.eB - 62);
+  };
+  for (int idx = threadIdx.x; idx < nf * 2 * NV * NF; idx += blockDim.x) {
+    const int p = idx % NF, fsv = idx / NF, vv = fsv % NV, side = fsv / NV % 2, fb = fsv / (2 * NV);
+    const int* e2 = sE + fb * 2 * NV + vv;
+    if (info[fb].bc != 0 || !far_below(e2[side * NV], e2[(1 - side) * NV])) continue;
+    int e, lf;
+    info[fb].side(side, e, lf);
+    const int r = lf >> 1, sn = r == 0 ? 1 : (r == 1 ? N : N * N);
+    const int s0 = r == 0 ? N : 1, s1 = r == 2 ? N : N * N;
+    const long long g = ((long long)e * NV + vv) * NM + ((lf & 1) ? P * sn : 0);
+    double s = 0.0;
+    for (int b = 0; b < (DIM == 3 ? N : 1); ++b) {
+      double row = 0.0;
+      for (int a = 0; a < N; ++a) {
+        const long long i = g + a * s0 + b * s1;
+        row = fma(B(p % Q, a), v ? fma(eps, v[i], u[i]) : u[i], row);
+      }
+      s = DIM == 3 ? fma(B(p / Q, b), row, s) : row;
+    }
+    fld[fb * stride + (side * NV + vv) * NF + p] = s;
+  }
+  __syncthreads();
+}
 
 // ------------------------------------------------------------ face kernel
 // One thread per (face, variable, line) in the transforms and one per face
@@ -257,7 +306,7 @@ __global__ void __maxnreg__(80) face_fix_kernel(
   double* sX = sm;                                   // [FPB][FX]
   double* sY = sX + FPB * A::FX;                     // [FPB][FY]
   FaceInfo* info = (FaceInfo*)(sY + FPB * A::FY);    // [FPB]
-  int* sE = (int*)(info + FPB);                      // [FPB][2][NV] coefficients of each side
+  int* sE = (int*)(info + FPB);                      // [FPB][2][NV] coefficients, both sides
   int* sS = sE + FPB * 2 * NV;                       // [FPB][3][NV] outputs f, T, S_n
   int* sT = sS + FPB * 3 * NV;                       // [FPB][NV] scaled tangential S
   const int f0 = blockIdx.x * FPB;
@@ -278,8 +327,9 @@ __global__ void __maxnreg__(80) face_fix_kernel(
     const double rmax = fmax(rA, rB);
     g.hn = 0.5 * rmax;
     const double one = 4611686018427387904.0;  // 2^62
-    fix_split(__double2ll_rn(rA / rmax * one), g.rhA[0], g.rhA[1]);
-    fix_split(__double2ll_rn(rB / rmax * one), g.rhB[0], g.rhB[1]);
+    const double less = fmin(rA, rB) / rmax;  // (one division: the larger's is 1)
+    fix_split(__double2ll_rn((rA < rB ? less : 1.0) * one), g.rhA[0], g.rhA[1]);
+    fix_split(__double2ll_rn((rA < rB ? 1.0 : less) * one), g.rhB[0], g.rhB[1]);
     const double c = (eR >= 0 ? 0.5 : 1.0) * ph.beta_s;
     g.ht[0] = 0.5 * geo[eL].rh[t0];
     g.ct[0] = fix_scale(c * geo[eL].rh[t0]);
@@ -306,20 +356,15 @@ __global__ void __maxnreg__(80) face_fix_kernel(
         m = max(m, fix_exp(val));
       }
       m = __reduce_max_sync(0xffffffffu, m);
-      if (lane == 0) {
-        sE[fb * 2 * NV + sv] = m;
-        // (a boundary face counts its side twice)
-        if (info[fb].bc != 0) sE[fb * 2 * NV + (1 - side) * NV + vv] = m;
-      }
+      if (lane == 0) sE[fb * 2 * NV + sv] = m;
     }
   }
   __syncthreads();
   // face coefficients per (face, variable, tangential mode): both sides'
   // values, their sum, and the sum of the normal derivatives scaled by 2/h_n
-  // over the larger of the two.  A side's values keep its own exponent (beside
-  // a neighbour 10^8 times larger one exponent for both left them 32 bits of
-  // the 53 that a double holds); the sums take the larger of the two.
+  // over the larger of the two (a boundary face counts its side twice)
   i64* C0 = (i64*)sY;
+  bool far = false;
   for (int idx = tid; idx < nf * NV * NT; idx += nth) {
     const int fb = idx / (NV * NT), rem = idx - fb * NV * NT;
     const int vv = rem / NT, l = rem - vv * NT;
@@ -329,8 +374,9 @@ __global__ void __maxnreg__(80) face_fix_kernel(
     const int s0 = r == 0 ? N : 1, s1 = r == 2 ? N : N * N;
     const int off = (DIM == 3 ? (l % N) * s0 + (l / N) * s1 : l * s0);
     int bad;
-    const int es[2] = {fix_emax(sE[(fb * 2) * NV + vv], bad), fix_emax(sE[(fb * 2 + 1) * NV + vv], bad)};
-    const int em = max(es[0], es[1]);
+    const int eA = sE[(fb * 2) * NV + vv], eB = sE[(fb * 2 + 1) * NV + vv];
+    const int em = fix_emax(max(eA, eB), bad);
+    far |= g.bc == 0 && far_below(min(eA, eB), max(eA, eB));
     i64 val[2] = {0, 0}, der[2] = {0, 0};
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
@@ -339,14 +385,13 @@ __global__ void __maxnreg__(80) face_fix_kernel(
       int xh[N], xl[N];
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        const i64 x = to_fix(src[k * sn], es[side], 59);
+        const i64 x = to_fix(src[k * sn], em, 59);
         if (k == (side == 0 ? P : 0)) val[side] = x;
         fix_split(x, xh[k], xl[k]);
       }
       // the side below has the face at its upper end
       const i64 d = fix_dot<N>(xh, xl, ft.dp[1 - side]);
-      der[side] = fix_shift(
-          side == 0 ? fix_mul(d, g.rhA[0], g.rhA[1]) : fix_mul(d, g.rhB[0], g.rhB[1]), em - es[side]);
+      der[side] = side == 0 ? fix_mul(d, g.rhA[0], g.rhA[1]) : fix_mul(d, g.rhB[0], g.rhB[1]);
     }
     if (g.eA < 0) {
       val[0] = val[1];
@@ -360,9 +405,9 @@ __global__ void __maxnreg__(80) face_fix_kernel(
     o[VALA * NV * NT] = val[0];
     o[VALB * NV * NT] = val[1];
     o[DN * NV * NT] = der[0] + der[1];
-    o[DT * NV * NT] = fix_shift(val[0], em - es[0]) + fix_shift(val[1], em - es[1]);
+    o[DT * NV * NT] = val[0] + val[1];
   }
-  __syncthreads();
+  const bool apart = __syncthreads_or(far);
   i64* C1 = (i64*)sX;  // 3-D: first tangential direction on its points, [4][NV][N][RQ]
   if constexpr (DIM == 3) {
     for (int idx = tid; idx < 4 * nf * NV * N; idx += nth) {
@@ -388,11 +433,8 @@ __global__ void __maxnreg__(80) face_fix_kernel(
     const int kind = idx / (nf * NV * NL), rem = idx - kind * nf * NV * NL;
     const int fb = rem / (NV * NL), vq = rem - fb * NV * NL;
     const int vv = vq / NL, q0 = vq - vv * NL;
-    int badA, badB;
-    const int esA = fix_emax(sE[(fb * 2) * NV + vv], badA), esB = fix_emax(sE[(fb * 2 + 1) * NV + vv], badB);
-    const int em = max(esA, esB);
-    const int bad = kind == VALA ? badA : (kind == VALB ? badB : badA | badB);
-    int se = (kind == VALA ? esA : (kind == VALB ? esB : em)) - 1022 - 59;
+    int bad;
+    int se = fix_emax(max(sE[(fb * 2) * NV + vv], sE[(fb * 2 + 1) * NV + vv]), bad) - 1022 - 59;
     int xh[N], xl[N];
     const i64* src;
     bool db;
@@ -404,8 +446,7 @@ __global__ void __maxnreg__(80) face_fix_kernel(
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         i64 x = src[k * RQ];
-        if (db)
-          x = fix_shift(x, em - esA) + fix_shift(src[k * RQ + (VALB - VALA) * NV * N * RQ], em - esB);
+        if (db) x += src[k * RQ + (VALB - VALA) * NV * N * RQ];
         fix_split(x, xh[k], xl[k]);
       }
     } else {
@@ -429,10 +470,12 @@ __global__ void __maxnreg__(80) face_fix_kernel(
 #pragma unroll
     for (int q = 0; q < Q; ++q) o[q * NL] = val[q];
   }
-  __syncthreads();
-  // fluxes, one thread per face point
   double* sP = DIM == 3 ? sY : sX;
   constexpr int PS = DIM == 3 ? A::FY : A::FX;
+  __syncthreads();
+  if (apart)
+    own_values<DIM, P, Q>(ft, info, sE, nf, u, v, v ? epsp[0] : 0.0, sP, PS);
+  // fluxes, one thread per face point
   double* gF = fflux;
   double* gS = fflux + (long long)F * NV * NF;  // [F][2][NV-1][NF]: T, S_n
   for (int idx = tid; idx < nf * NF; idx += nth) {
@@ -736,9 +779,10 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
   double* s1 = sm + ASZ;                        // DIM arrays: derivatives, fluxes, G_r
   struct ElFace {
     int f;           // face id
-    FixScale c0, c1; // 2/h_r; (2/h_r)^2 c beta_s
+    FixMag c0;       // 2/h_r
+    FixScale c1;     // (2/h_r)^2 c beta_s
   };
-  static_assert(sizeof(ElFace) <= 36, "vol_bytes");
+  static_assert(sizeof(ElFace) <= 32, "vol_bytes");
   ElFace* ef = (ElFace*)(s1 + DIM * ASZ);       // [EPB][2 DIM]
   int* sE = (int*)(ef + EPB * 2 * DIM);         // [EPB][NV] coefficients
   int* sH = sE + EPB * NV;                      // [EPB][NV] fluxes and face data
@@ -756,7 +800,7 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
       ElFace x;
       x.f = eface[(long long)(e0 + eb) * 2 * DIM + lf];
       const double rh = geo[e0 + eb].rh[lf >> 1];
-      x.c0 = fix_scale(rh);
+      x.c0 = fix_mag(rh);
       x.c1 = fix_scale(rh * rh * ph.beta_s * (faces[(long long)x.f * 6 + 2] >= 0 ? 0.5 : 1.0));
       ef[j] = x;
     }

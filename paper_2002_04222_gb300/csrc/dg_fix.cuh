@@ -16,6 +16,7 @@
 // in the inputs mark the (element, variable) bad: everything converted back
 // from it is NaN.
 #pragma once
+#include <algorithm>
 #include <cstring>
 #include "dg_internal.h"
 
@@ -73,7 +74,7 @@ constexpr i64 FIX_HALF = 1ll << 29;
 // x / 2^sh to the nearest, for any sh >= 0 and |x| < 2^61: from 62 on that is 0
 // (and 2^63, twice the half unit to add at 63, is not an i64)
 DG_HD i64 fix_shift(i64 x, int sh) {
-  sh = sh < 62 ? sh : 62;
+  sh = std::min(sh, 62);
   return (x + ((1ll << sh) >> 1)) >> sh;
 }
 
@@ -89,31 +90,39 @@ DG_HD void fix_split(i64 x, int& h, int& l) {
 DG_HD i64 to_fix(double v, int emax, int nb) {
   const int hi = fix_hi(v);
   const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | fix_lo(v);
-  int d = emax - ((hi >> 20) & 0x7ff);
-  d = d < 63 ? d : 63;
+  const int d = std::min(emax - ((hi >> 20) & 0x7ff), 63);
   const i64 a = (i64)((m << (nb - 53)) >> d), s = (i64)(hi >> 31);
   return (a ^ s) - s;
 }
 
-// A factor of magnitude rm 2^(er - 62), 2^61 <= rm < 2^62 (0: rm = 0), its sign
-// kept apart: what is multiplied is a magnitude, cut off towards 0 on both
-// sides (a negative rm would cut its products off towards -infinity and turn
-// zeros into -1)
-struct FixScale {
+// A positive factor rm 2^(er - 62), 2^61 <= rm < 2^62 (0: rm = 0)
+struct FixMag {
   int h, l;  // balanced halves of rm
   int er;
+};
+// and one of either sign, kept apart: what is multiplied is a magnitude, cut
+// off towards 0 on both sides (a negative rm would cut its products off towards
+// -infinity and turn zeros into -1)
+struct FixScale : FixMag {
   int sg;    // 0 or -1
 };
-DG_HD FixScale fix_scale(double r) {
-  FixScale f;
+DG_HD FixMag fix_mag(double r) {
+  FixMag f;
   const int hi = fix_hi(r), E = (hi >> 20) & 0x7ff;
   i64 m = (i64)(((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | fix_lo(r)) << 9;
   if (E == 0) m = 0;
   fix_split(m, f.h, f.l);
   f.er = E == 0 ? -4000 : E - 1022;
-  f.sg = hi >> 31;
   return f;
 }
+DG_HD FixScale fix_scale(double r) {
+  FixScale f;
+  static_cast<FixMag&>(f) = fix_mag(r);
+  f.sg = fix_hi(r) >> 31;
+  return f;
+}
+DG_HD int fix_sign(const FixMag&) { return 0; }
+DG_HD int fix_sign(const FixScale& f) { return f.sg; }
 
 // x rm / 2^62
 DG_HD i64 fix_mul(i64 x, int rh, int rl) {
@@ -124,15 +133,15 @@ DG_HD i64 fix_mul(i64 x, int rh, int rl) {
 }
 
 // v r as an integer below 2^nb (nb <= 60); emax >= exponent(v) + r.er
-DG_HD i64 to_fix_mul(double v, const FixScale& r, int emax, int nb) {
+template <class R>
+DG_HD i64 to_fix_mul(double v, const R& r, int emax, int nb) {
   const int hi = fix_hi(v);
   const u64 m = ((u64)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | fix_lo(v);
   const int E = (hi >> 20) & 0x7ff;
   i64 a = fix_mul((i64)(m << 7), r.h, r.l);
-  int d = emax - E - r.er + 60 - nb;
-  d = E == 0 || d > 63 ? 63 : d;
+  const int d = E == 0 ? 63 : std::min(emax - E - r.er + 60 - nb, 63);
   a >>= d;
-  const i64 s = (i64)((hi >> 31) ^ r.sg);
+  const i64 s = (i64)((hi >> 31) ^ fix_sign(r));
   return (a ^ s) - s;
 }
 

@@ -36,6 +36,10 @@ struct FaceInfoGen {
   int eA, fA, eB, fB;  // owner and neighbour (-1: none) and their local faces
   int bc;              // boundary type (0: interior)
   FixScale cb;         // c beta_s
+  __device__ __forceinline__ void side(int s, int& e, int& lf) const {
+    e = s == 0 ? eA : eB;
+    lf = s == 0 ? fA : fB;
+  }
 };
 static_assert(sizeof(FaceInfoGen) <= 64, "face_bytes");
 
@@ -162,9 +166,9 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     }
   }
   __syncthreads();
-  // per side, at its own exponent: the face's coefficients and those of the
-  // normal derivative
+  // per side: the face's coefficients and those of the normal derivative
   i64* C0 = (i64*)sY;  // [2 side][2][NV][NT]
+  bool far = false;
   for (int idx = tid; idx < nf * 2 * NV * NT; idx += nth) {
     const int fb = idx / (2 * NV * NT), rem = idx - fb * 2 * NV * NT;
     const int sv = rem / NT, l = rem - sv * NT, side = sv / NV, vv = sv - side * NV;
@@ -176,7 +180,9 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     const double* src = sX + fb * A::GX + sv * NM +
                         (DIM == 3 ? (l % N) * s0 + (l / N) * s1 : l * s0);
     int bad, xh[N], xl[N];
-    const int em = fix_emax(sE[fb * 2 * NV + sv], bad);
+    const int eA = sE[(fb * 2) * NV + vv], eB = sE[(fb * 2 + 1) * NV + vv];
+    const int em = fix_emax(max(eA, eB), bad);
+    far |= g.bc == 0 && far_below(min(eA, eB), max(eA, eB));
     i64 first = 0, last = 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
@@ -189,7 +195,7 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     o[0] = (lf & 1) ? last : first;
     o[NV * NT] = (lf & 1) ? fix_dot<N>(xh, xl, ft.dp[1]) : fix_dot<N>(xh, xl, ft.dp[0]);
   }
-  __syncthreads();
+  const bool apart = __syncthreads_or(far);
   // 3-D, first tangential direction: per side B and DB on the values, B on the
   // normal derivative
   i64* C1 = (i64*)sX;  // [2 side][3][NV][N][RQ]
@@ -213,8 +219,8 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     __syncthreads();
   }
   // last tangential direction: fields [NFLD][NV][NF], the values as doubles,
-  // the derivatives as integers of one scale (both sides' too): 0, 1 values;
-  // 2 + DIM side + (0 normal, 1.. tangential)
+  // the derivatives as integers of one scale: 0, 1 values; 2 + DIM side + (0
+  // normal, 1.. tangential)
   const int eT = max(ft.edp + ft.eB, ft.eDB) + (DIM == 3 ? ft.eB : 0);
   for (int idx = tid; idx < A::NFLD * nf * NV * NL; idx += nth) {
     const int kind = idx / (nf * NV * NL), rem = idx - kind * nf * NV * NL;
@@ -242,22 +248,22 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
       for (int q = 0; q < Q; ++q) y[q] = fix_dot<N>(xh, xl, ft.B + q * N);
     }
     double* o = (DIM == 3 ? sY + fb * A::GY : sX + fb * A::GX) + (kind * NV + vv) * NF + q0;
-    int bad;
-    const int es = fix_emax(sE[(fb * 2 + side) * NV + vv], bad);
     if (kind < 2) {
-      const int se = es - 1022 - 59 + (DIM - 1) * ft.eB;
+      int bad;
+      const int se = fix_emax(max(sE[(fb * 2) * NV + vv], sE[(fb * 2 + 1) * NV + vv]), bad) - 1022 -
+                     59 + (DIM - 1) * ft.eB;
 #pragma unroll
       for (int q = 0; q < Q; ++q) o[q * NL] = fix_to_double(y[q], se, bad);
     } else {
-      int other;
-      sh += max(fix_emax(sE[(fb * 2 + 1 - side) * NV + vv], other) - es, 0);
 #pragma unroll
       for (int q = 0; q < Q; ++q) ((i64*)o)[q * NL] = fix_shift(y[q], sh);
     }
   }
-  __syncthreads();
   double* sP = DIM == 3 ? sY : sX;
   constexpr int PS = DIM == 3 ? A::GY : A::GX;
+  __syncthreads();
+  if (apart)
+    own_values<DIM, P, Q>(ft, info, sE, nf, u, v, v ? epsp[0] : 0.0, sP, PS);
   double* gS = fflux + (long long)F * NV * NF;  // [E][2 DIM][2][NV-1][NF]
   for (int idx = tid; idx < nf * NF; idx += nth) {
     const int fb = idx / NF, p = idx - fb * NF;
@@ -271,7 +277,7 @@ __global__ void __launch_bounds__(256, 2) face_gen_kernel(
     // exponent, both sides' products in one sum
     double dQ[DIM][NV];
     const double Jf = fd[DIM * NF] * ft.iw[p % Q] * (DIM == 3 ? ft.iw[p / Q] : 1.0);
-    const FixScale sJ = fix_scale(Jf);
+    const FixMag sJ = fix_mag(Jf);
     {
       const double* gA = gg.fgeo + ((long long)g.eA * 2 * DIM + g.fA) * DIM * DIM * NF + p;
       const double* gB = interior ? gg.fgeo + ((long long)g.eB * 2 * DIM + g.fB) * DIM * DIM * NF + p : gA;
@@ -709,8 +715,8 @@ __global__ void __launch_bounds__(256, 2) vol_gen_kernel(
     const int off = eb * NV * VP + q + (RQ - Q) * (q / Q);
     const double* gp = gg.vgeo + (long long)(e0 + eb) * (DIM * DIM + 1) * NQ + q;
     const int qx = q % Q, qy = (q / Q) % Q, qz = q / (Q * Q);
-    const FixScale sJ =
-        fix_scale(gp[DIM * DIM * NQ] * ft.iw[qx] * ft.iw[qy] * (DIM == 3 ? ft.iw[qz] : 1.0));
+    const FixMag sJ =
+        fix_mag(gp[DIM * DIM * NQ] * ft.iw[qx] * ft.iw[qy] * (DIM == 3 ? ft.iw[qz] : 1.0));
     int gbad, ch[DIM][DIM], cl[DIM][DIM];
     const int eg = fix_emax(sG[eb], gbad);
 #pragma unroll
