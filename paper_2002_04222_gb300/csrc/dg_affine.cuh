@@ -27,31 +27,6 @@
 
 namespace dg {
 
-template <int DIM, int P, int Q>
-struct Aff {
-  using C = Cfg<DIM, P, Q>;
-  static constexpr int N = P + 1, NV = DIM + 2, NM = C::NM, NQ = C::NQ, NF = C::NF;
-  // rows along direction 0 padded to an odd length: lines along it start in
-  // different shared-memory banks
-  static constexpr int RQ = Q | 1;
-  static constexpr int Q2 = DIM == 3 ? Q : 1, N2 = DIM == 3 ? N : 1;
-  static constexpr int VP = RQ * Q * Q2;      // padded volume array of one variable
-  static constexpr int LQ = NF;               // lines of one direction on the Gauss grid
-  // volume kernel, per element: DIM + 1 arrays
-  static constexpr int VOL_EL = (DIM + 1) * NV * VP;
-  // face kernel, per face: two regions used in turn
-  static constexpr int NT = DIM == 3 ? N * N : N;   // coefficients of a face
-  static constexpr int KK = DIM + 2;                // trace fields: both values, d_n, d_t
-  static constexpr int imax(int a, int b) { return a > b ? a : b; }
-  static constexpr int FX = imax(2 * NV * NM, DIM == 3 ? 4 * NV * N * RQ : KK * NV * NF);
-  static constexpr int FY = imax(4 * NV * NT, DIM == 3 ? KK * NV * NF : 0);
-  // shared memory in bytes of `e` elements / `f` faces per block
-  static constexpr size_t vol_bytes(int e) {
-    return (size_t)e * (8 * VOL_EL + 2 * DIM * 32 + 4 * NV * 4);
-  }
-  static constexpr size_t face_bytes(int f) { return (size_t)f * (8 * (FX + FY) + 128 + 6 * NV * 4); }
-};
-
 // ------------------------------------------------------------ pointwise fluxes
 // H~_r = rh_r (F_r - G_r) at a volume point; dU[r] are reference derivatives
 // (the physical ones are rh_r dU[r]).  One reciprocal; rh and mu ride on
@@ -1019,10 +994,7 @@ __global__ void __launch_bounds__(256, 2) vol_fix_kernel(
 template <int DIM, int P, int Q>
 dg_status launch_fix(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
   using A = Aff<DIM, P, Q>;
-  constexpr size_t cap = 227 * 1024;
-  int epb = m->tune.vol_epb, fpb = m->tune.lift_epb * DIM;
-  while (epb > 1 && A::vol_bytes(epb) > cap) --epb;
-  while (fpb > 1 && A::face_bytes(fpb) > cap) --fpb;
+  const int epb = m->tune.vol_epb, fpb = m->tune.lift_epb * DIM;
   const size_t vsm = A::vol_bytes(epb), fsm = A::face_bytes(fpb);
   if (!a.skip_face) {
     DG_CUDA(cudaFuncSetAttribute(face_fix_kernel<DIM, P, Q>,

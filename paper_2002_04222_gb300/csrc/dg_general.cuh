@@ -17,21 +17,6 @@
 
 namespace dg {
 
-template <int DIM, int P, int Q>
-struct Gen : Aff<DIM, P, Q> {
-  using A = Aff<DIM, P, Q>;
-  static constexpr int NFLD = 2 + 2 * DIM;  // trace fields: both values, both sides' derivatives
-  static constexpr int GX = A::imax(2 * A::NV * A::NM, DIM == 3 ? 6 * A::NV * A::N * A::RQ
-                                                                : NFLD * A::NV * A::NF);
-  static constexpr int GY = A::imax(4 * A::NV * A::NT, DIM == 3 ? NFLD * A::NV * A::NF : 0);
-  static constexpr size_t vol_bytes(int e) {
-    return (size_t)e * (8 * A::VOL_EL + 2 * DIM * 4 + (5 * A::NV + 1) * 4 + 16) + 4 * A::NM;
-  }
-  static constexpr size_t face_bytes(int f) {
-    return (size_t)f * (8 * (GX + GY) + 64 + (2 + 1 + 1 + 4) * A::NV * 4 + 16);
-  }
-};
-
 struct FaceInfoGen {
   int eA, fA, eB, fB;  // owner and neighbour (-1: none) and their local faces
   int bc;              // boundary type (0: interior)
@@ -959,10 +944,7 @@ dg_status launch_minv_exp(dg_mesh_s* m, cudaStream_t s) {
 template <int DIM, int P, int Q>
 dg_status launch_gen(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
   using A = Gen<DIM, P, Q>;
-  constexpr size_t cap = 227 * 1024;
-  int epb = m->tune.vol_epb, fpb = m->tune.lift_epb * DIM;
-  while (epb > 1 && A::vol_bytes(epb) > cap) --epb;
-  while (fpb > 1 && A::face_bytes(fpb) > cap) --fpb;
+  const int epb = m->tune.vol_epb, fpb = m->tune.lift_epb * DIM;
   const size_t vsm = A::vol_bytes(epb), fsm = A::face_bytes(fpb);
   const GenGeo gg = gen_geo(m);
   if (!a.skip_face) {

@@ -452,24 +452,29 @@ static void default_tune(dg_mesh_s* m) {
   if (DIM == 3 && m->tune.lift_threads < 128) m->tune.lift_threads = 128;
 }
 
-// candidate (elements per CTA, threads per CTA) launch shapes of the
-// sum-factorisation kernels that fit the shared memory of one CTA
-template <int DIM, int P, int Q>
-static void tune_candidates(std::vector<int2>& vol, std::vector<int2>& lift) {
-  using C = Cfg<DIM, P, Q>;
+// candidate (elements per CTA, threads per CTA) launch shapes whose shared
+// memory one CTA can have; lift: the face kernel's, DIM faces an element
+template <int DIM, class A>
+static void tune_candidates_of(std::vector<int2>& vol, std::vector<int2>& lift) {
   const int epbs3[] = {1, 2, 3, 4};
   const int epbs2[] = {1, 2, 4, 8, 16, 32};
   // every warp multiple up to the kernels' bound: a count just above the
   // Gauss points of one or more elements (224 for 216 at Q = 6) gives the
   // per-point flux stage one pass without idle lanes
   const int nts[] = {64, 96, 128, 160, 192, 224, 256};
-  const size_t cap = 200 * 1024;
   for (int e : (DIM == 3 ? std::vector<int>(epbs3, epbs3 + 4) : std::vector<int>(epbs2, epbs2 + 6)))
     for (int t : nts) {
       if (DIM == 3 && t < 128) continue;
-      if (sizeof(double) * C::vol_sm(e) <= cap) vol.push_back(make_int2(e, t));
-      if (sizeof(double) * C::lift_sm(e) <= cap) lift.push_back(make_int2(e, t));
+      if (A::vol_bytes(e) <= FIX_SMEM) vol.push_back(make_int2(e, t));
+      if (A::face_bytes(e * DIM) <= FIX_SMEM) lift.push_back(make_int2(e, t));
     }
+}
+template <int DIM, int P, int Q>
+static void tune_candidates(const dg_mesh_s* m, std::vector<int2>& vol, std::vector<int2>& lift) {
+  if (m->curved)
+    tune_candidates_of<DIM, Gen<DIM, P, Q>>(vol, lift);
+  else
+    tune_candidates_of<DIM, Aff<DIM, P, Q>>(vol, lift);
 }
 
 template <int DIM, int P, int Q, bool CV>
@@ -578,7 +583,7 @@ dg_status launch_project(dg_mesh_s* m, int what, double t, double* out, cudaStre
 template <int DIM, int P, int Q>
 static dg_status run_autotune(dg_mesh_s* m, int reps, dg_tune_result* res, cudaStream_t s) {
   std::vector<int2> vc, lc;
-  tune_candidates<DIM, P, Q>(vc, lc);
+  tune_candidates<DIM, P, Q>(m, vc, lc);
   // a valid state to time on: the projected analytic field
   DG_TRY(launch_project(m, 0, 0.0, m->w1, s));
   EvalArgs a{};
@@ -624,7 +629,6 @@ static dg_status run_autotune(dg_mesh_s* m, int reps, dg_tune_result* res, cudaS
   res->vol_ms_default = dflt;
   m->tune.vol_epb = t.vol_epb;
   m->tune.vol_threads = t.vol_threads;
-  run_residual<DIM, P, Q>(m, a, s);  // traces and fluxes for the lift timing
   best = 1e30;
   dflt = -1.0;
   for (const int2& c : lc) {
@@ -676,7 +680,7 @@ bool tune_valid(dg_mesh_s* m, const dg_tune_result* t) {
 #define DG_RUN(D_, P_, Q_)                                                            \
   if (m->dim == D_ && m->P == P_ && m->Q == Q_) {                                     \
     std::vector<int2> vc, lc;                                                         \
-    tune_candidates<D_, P_, Q_>(vc, lc);                                              \
+    tune_candidates<D_, P_, Q_>(m, vc, lc);                                            \
     bool v = false, l = false;                                                        \
     for (const int2& c : vc) v |= c.x == t->vol_epb && c.y == t->vol_threads;         \
     for (const int2& c : lc) l |= c.x == t->lift_epb && c.y == t->lift_threads;       \
