@@ -153,6 +153,9 @@ dg_status dg_mesh_create(const dg_mesh_desc* mesh, const dg_physics* phys, void*
                          dg_mesh_t* out);
 dg_status dg_mesh_destroy(dg_mesh_t m);
 dg_status dg_mesh_info(dg_mesh_t m, dg_mesh_info_t* info);
+/* 1 if the mesh takes the general-geometry kernels, 0 if the axis-aligned ones
+ * (launch shapes of the one kind say nothing about the other), or DG_ERR_ARG. */
+int dg_mesh_general(dg_mesh_t m);
 
 /* Autotuning of the sum-factorisation kernels (no counterpart in the paper,
  * whose kernels ran on CPUs): dg_autotune times every launch shape (elements

@@ -319,8 +319,15 @@ def autotune(mesh, reps=5, stream=None):
     return {f: getattr(r, f) for f, _ in _lib.TuneResult._fields_}
 
 
+def tuning_key(mesh):
+    """The tuning table's key of a mesh: (dim, P, Q) and the kind of kernels it takes
+    (rotated and sheared straight elements take the curved ones')."""
+    return (f"{mesh.info['dim']}d_P{mesh.info['P']}_Q{mesh.info['Q']}"
+            + ("_general" if lib().dg_mesh_general(mesh.handle) == 1 else ""))
+
+
 def apply_tuning(mesh, table_path=TUNING_TABLE):
-    """Apply the stored tuning-table entry of this mesh's (dim, P, Q), if any.
+    """Apply the stored tuning-table entry of this mesh's key (tuning_key), if any.
     The shapes that fill the GPU differ with the mesh: an entry that names the
     element count it was tuned on (n_elem) serves meshes within a factor of 4
     of it, and the closest one is taken; others keep the built-in rule."""
@@ -329,10 +336,7 @@ def apply_tuning(mesh, table_path=TUNING_TABLE):
     import os
     if not os.path.exists(table_path):
         return None
-    key = f"{mesh.info['dim']}d_P{mesh.info['P']}_Q{mesh.info['Q']}"
-    if mesh._desc.geom_order == 2:
-        key += "_general"
-    entries = json.load(open(table_path)).get(key)
+    entries = json.load(open(table_path)).get(tuning_key(mesh))
     if entries is None:
         return None
     off = lambda e: abs(math.log(mesh.info["n_elem"] / e["n_elem"])) if "n_elem" in e else 0.0

@@ -138,6 +138,7 @@ SIGNATURES = {
 }
 # those that return a value of their own (an int) instead of a status
 VALUES = {
+    "dg_mesh_general": [VP],
     "dg_precond_wait_limit": [VP, I],
 }
 

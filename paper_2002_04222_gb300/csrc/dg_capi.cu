@@ -530,6 +530,8 @@ dg_status dg_mesh_info(dg_mesh_t m, dg_mesh_info_t* info) {
   return DG_OK;
 }
 
+int dg_mesh_general(dg_mesh_t m) { return m ? m->curved : DG_ERR_ARG; }
+
 dg_status dg_autotune(dg_mesh_t m, int reps, dg_tune_result* result, void* stream) {
   if (!m || !result || reps < 1) return DG_ERR_ARG;
   dg_tune_result r{};

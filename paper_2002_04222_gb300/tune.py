@@ -34,9 +34,7 @@ def main(reps=20):
     table = {}
     for c in cases():
         m = dgl.Mesh.from_case(c)
-        key = f"{m.info['dim']}d_P{m.info['P']}_Q{m.info['Q']}"
-        if c.mesh.geom_order == 2:   # curved elements have kernels of their own
-            key += "_general"
+        key = dgl.tuning_key(m)
         r = dgl.autotune(m, reps=reps)
         r["workload"] = c.name
         r["n_elem"] = m.info["n_elem"]

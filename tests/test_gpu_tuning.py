@@ -40,3 +40,22 @@ def test_shapes_that_fit_the_launched_kernels_are_candidates(dgl, make, accepted
         assert torch.equal(m.residual(u), r), (ve, le)
     for ve, le in refused:
         assert tune(ve, le) == DG_ERR_ARG, (ve, le)
+
+
+@pytest.mark.parametrize("make,general", [
+    (lambda: w.small_tgv_case((2, 2, 2), P=2), False),
+    (lambda: w.rotated_box_case((2, 2, 2), P=2), True),              # straight, not boxes
+    (lambda: w.rotated_box_case((2, 2, 2), P=2, order=2), True),
+    (lambda: w.wavy_box_case((2, 2, 2), P=2), True),
+])
+def test_a_mesh_takes_the_entry_of_its_own_kernels(dgl, tmp_path, make, general):
+    import json
+    c = make()
+    m = dgl.Mesh.from_case(c)
+    assert dgl.lib().dg_mesh_general(m.handle) == int(general)
+    assert dgl.lib().dg_mesh_general(None) == DG_ERR_ARG
+    entry = dict(vol_threads=128, lift_threads=128)
+    table = tmp_path / "t.json"
+    table.write_text(json.dumps({"3d_P2_Q5": dict(entry, vol_epb=1, lift_epb=1),
+                                 "3d_P2_Q5_general": dict(entry, vol_epb=2, lift_epb=2)}))
+    assert dgl.apply_tuning(m, str(table))["vol_epb"] == 1 + general
