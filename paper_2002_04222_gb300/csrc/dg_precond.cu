@@ -446,32 +446,45 @@ __global__ void __launch_bounds__(128) brj_tracejac_gen_kernel(
 // q0 per (j,a) accumulated by the types of direction 1, then q1.  The own-side
 // trace term adds, on each face, the face-slice modes (vertex mode across the
 // face) contracted over the two (one) tangential face-point directions.
-// the FP64 form of a mass-matrix row, out of line: inlined, the compiler
-// predicates its few instructions instead of branching round them and the FP64
-// pipe is as busy as before
 template <int N, typename T>
-__device__ __noinline__ T fp64_row(const double* m, const T* x, int str) {
+__device__ __forceinline__ T fp64_row(const double* m, const T* x, int str) {
   double s = 0.0;
 #pragma unroll
   for (int k = 0; k < N; ++k) s += m[k] * (double)x[k * str];
   return (T)s;
 }
 template <typename T>
-__device__ __noinline__ T fp64_scaled(double sc, T x, double add) {
+__device__ __forceinline__ T fp64_scaled(double sc, T x, double add) {
   return (T)__dadd_rn(__dmul_rn(sc, (double)x), add);
 }
+// out of line for the values that float pairs cannot decide (PairSum): inlined
+// there, the FP64 pipe is as busy as without the pairs
+template <int N, typename T>
+__device__ __noinline__ T fp64_row_call(const double* m, const T* x, int str) {
+  return fp64_row<N>(m, x, str);
+}
+__device__ __noinline__ float fp64_scaled_call(double sc, float x, double add) {
+  return fp64_scaled(sc, x, add);
+}
 
-// shared-memory layout of the block assembly
-template <int DIM, int P, int Q>
+// shared-memory layout of the block assembly (sizes in T)
+template <int DIM, int P, int Q, typename T>
 struct BlockSmem {
-  static constexpr int N = P + 1, N2 = N * N, NM = DIM == 3 ? N2 * N : N2;
+  static constexpr int N = P + 1, N2 = N * N, NM = DIM == 3 ? N2 * N : N2, NQ = DIM == 3 ? Q * Q * Q : Q * Q;
   // n1 stride of T2: N N2 values, padded (from N = 4 on) to N2 modulo 32
   static constexpr int T2N = N * N2 + (N >= 4 ? ((N2 - N * N2) % 32 + 32) % 32 : 0);
   static constexpr int imax(int a, int b) { return a > b ? a : b; }
   // (the trace term uses both for the faces' Jacobians and half contractions)
   static constexpr int T1SZ = DIM == 3 ? 6 * N2 * Q * Q : 4 * N2 * Q;
   static constexpr int T2SZ = DIM == 3 ? imax(Q * N * T2N, 6 * N2 * Q) : 0;
-  static constexpr int XS = DIM == 3 && NM % 32 == 0 ? NM + 8 : NM;  // row stride of X and Y
+  // row stride of X and Y: n0 falls 8 banks apart
+  static constexpr int XS = DIM == 3 && NM % 32 == 0 ? NM + 32 / (int)sizeof(T) : NM;
+  // 3-D: T1 behind the factors' products in Y, which is free until the
+  // mass-matrix step, wherever they fit: FP64 blocks at P = 3, Q = 6 take 106 KB
+  // so and two of them share an SM (with T1 of its own 133 KB, one: assembly of
+  // 10^3 blocks 17.2 ms against 16.4 with the former layouts)
+  static constexpr bool T1_IN_Y = DIM == 3 && 4 * Q * N2 + T1SZ <= NM * XS;
+  static constexpr int SCRATCH = NQ * DIM * (DIM + 1) + (T1_IN_Y ? 0 : T1SZ) + T2SZ;  // sW, T1, T2
 };
 
 // FP32 results of FP64 arithmetic without the FP64 pipe.  A sum of products
@@ -507,8 +520,17 @@ struct PairSum {
   }
 };
 
+// blocks per SM: FP32 up to P = 3 three; the smallest elements' blocks are a few
+// values a thread and wait on one another, so more of them (2-D P = 2, 32x32
+// elements: 94 us at 32 registers, 143 at 53)
+template <int DIM, int P, typename T>
+constexpr int block_residency() {
+  if (DIM == 2 ? P <= 2 : P == 1) return sizeof(T) == 4 || (DIM == 2 && P == 1) ? 8 : 6;
+  return sizeof(T) == 4 && P <= 3 ? 3 : 1;
+}
+
 template <int DIM, int P, int Q, typename T, bool CV>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 && P <= 3 ? 3 : 1) brj_block_kernel(
+__global__ void __launch_bounds__(256, block_residency<DIM, P, T>()) brj_block_kernel(
     const __grid_constant__ Tables tab, const ElemGeo* __restrict__ geo,
     const double* __restrict__ minv, int e_begin, const T* __restrict__ W,
     const T* __restrict__ Jd, double dta, T* __restrict__ blocks, int ld) {
@@ -519,17 +541,21 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && P <= 3 ? 3 : 1) brj_blo
   constexpr int N2 = N * N;
   // 3-D: T1 [up to 6 (j,a) of a type][Q*Q][N2], T2 [Q][N n1][N m1][N2]
   // per type; 2-D: T1 [4][N2][Q]
-  using BS = BlockSmem<DIM, P, Q>;
+  using BS = BlockSmem<DIM, P, Q, T>;
   constexpr int T1SZ = BS::T1SZ, T2SZ = BS::T2SZ, T2N = BS::T2N, T2Q = N * T2N, XS = BS::XS;
+  // float pairs where a row is long enough to pay for them
+  constexpr bool PAIRS = std::is_same<T, float>::value && N >= (DIM == 3 ? 3 : 4);
+  // (3-D P = 2 FP64 blocks: 1.81 ms out of line, 1.95 inline; the others equal)
+  constexpr bool CALL = std::is_same<T, double>::value && DIM == 3 && N == 3;
   __shared__ T sB1[Q * N], sD1[Q * N];
   __shared__ double sMi[N * N];
-  __shared__ float sMh[N * N], sMl[N * N];
+  __shared__ float sMh[PAIRS ? N * N : 1], sMl[PAIRS ? N * N : 1];
   extern __shared__ unsigned char smraw[];
   T* X = reinterpret_cast<T*>(smraw);           // [NM (col n)][XS (row m)]
   T* Y = X + NM * XS;
   T* sW = Y + NM * XS;                          // [JA][NQ]; later the dense M^-1, over T1 and T2 too
-  T* T1 = sW + JA * NQ;
-  T* T2 = T1 + T1SZ;
+  T* T1 = BS::T1_IN_Y ? Y + 4 * Q * N2 : sW + JA * NQ;
+  T* T2 = BS::T1_IN_Y ? sW + JA * NQ : T1 + T1SZ;
   const int el = blockIdx.x, e = e_begin + el;
   const int k = blockIdx.y / NV, l = blockIdx.y % NV;
   for (int i = threadIdx.x; i < Q * N; i += blockDim.x) {
@@ -541,13 +567,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && P <= 3 ? 3 : 1) brj_blo
   }
   for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
     sMi[i] = tab.Minv[i];
-    sMh[i] = (float)tab.Minv[i];
-    sMl[i] = (float)(tab.Minv[i] - (double)(float)tab.Minv[i]);
+    if constexpr (PAIRS) {
+      sMh[i] = (float)tab.Minv[i];
+      sMl[i] = (float)(tab.Minv[i] - (double)(float)tab.Minv[i]);
+    }
   }
   const T* We = W + (long long)el * NQ * NW;
   for (int i = threadIdx.x; i < NQ * JA; i += blockDim.x)
     sW[i] = We[(long long)(k * NV + l) * JA * NQ + i];  // contiguous slice of (k, l)
-  for (int i = threadIdx.x; i < T1SZ + T2SZ; i += blockDim.x) T1[i] = (T)0;
+  for (int i = threadIdx.x; i < T1SZ; i += blockDim.x) T1[i] = (T)0;
+  for (int i = threadIdx.x; i < T2SZ; i += blockDim.x) T2[i] = (T)0;
   __syncthreads();
   // factor of direction r for test (F) / trial (G) side of combination (j, a)
   auto ftab = [&](int j, int r) -> const T* { return r == j ? sD1 : sB1; };
@@ -797,15 +826,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && P <= 3 ? 3 : 1) brj_blo
       const int base = m - mc[ax] * str;
       const T* x = src + col * XS + base;
       T val;
-      bool done = false;
-      if constexpr (std::is_same<T, float>::value) {
+      if constexpr (PAIRS) {
         PairSum ps;
 #pragma unroll
         for (int kk = 0; kk < N; ++kk) ps.add(sMh[mc[ax] * N + kk], sMl[mc[ax] * N + kk], x[kk * str]);
         val = ps.value();
-        done = !ps.near(val);
+        if (ps.near(val)) val = fp64_row_call<N>(sMi + mc[ax] * N, x, str);
+      } else {
+        val = CALL ? fp64_row_call<N>(sMi + mc[ax] * N, x, str) : fp64_row<N>(sMi + mc[ax] * N, x, str);
       }
-      if (!done) val = fp64_row<N>(sMi + mc[ax] * N, x, str);
       dst[col * XS + m] = val;
     }
     __syncthreads();
@@ -820,17 +849,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && P <= 3 ? 3 : 1) brj_blo
   for (int i = threadIdx.x; i < NM * NM; i += blockDim.x) {
     const int n = i / NM, m = i % NM;
     const T x = src[n * XS + m];
+    const double one = k == l && m == n ? 1.0 : 0.0;
     T v;
-    bool done = false;
-    if constexpr (std::is_same<T, float>::value) {
-      if (!(k == l && m == n)) {
-        PairSum ps;
-        ps.add(sh, sl, x);
-        v = ps.value();
-        done = !ps.near(v);
-      }
+    if constexpr (PAIRS) {
+      PairSum ps;
+      ps.add(sh, sl, x);
+      v = ps.value();
+      if (one != 0.0 || ps.near(v)) v = fp64_scaled_call(sc, x, one);
+    } else {
+      v = fp64_scaled(sc, x, one);
     }
-    if (!done) v = fp64_scaled(sc, x, k == l && m == n ? 1.0 : 0.0);
     // stored transposed: the inverse of the transpose is the transpose of the
     // inverse, which the column-streaming block GEMV reads
     out[(long long)(l * NM + n) * ld + k * NM + m] = v;
@@ -1291,11 +1319,12 @@ struct BRJImpl {
     DG_CUDA(cudaFuncSetAttribute(brj_weights_kernel<DIM, P, Q, T, CV>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm));
     // general elements stage the dense M^-1 beside the weights
-    const int wsz = NQ * DIM * (DIM + 1);
-    using BS = BlockSmem<DIM, P, Q>;
-    constexpr int TSZ = BS::T1SZ + BS::T2SZ;
-    const int scratch = wsz + TSZ;
-    const size_t bsm = sizeof(T) * (2 * NM * BS::XS + (CV && NM * NM > scratch ? NM * NM : scratch));
+    using BS = BlockSmem<DIM, P, Q, T>;
+    static_assert(!(std::is_same<T, double>::value && DIM == 3 && P == 3) ||
+                      sizeof(T) * (2 * NM * BS::XS + BS::SCRATCH) <= 112 * 1024,
+                  "two FP64 P = 3 blocks share an SM");
+    const size_t bsm =
+        sizeof(T) * (2 * NM * BS::XS + (CV && NM * NM > BS::SCRATCH ? NM * NM : BS::SCRATCH));
     DG_CUDA(cudaFuncSetAttribute(brj_block_kernel<DIM, P, Q, T, CV>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm));
     const int CH = pc->wchunk;
