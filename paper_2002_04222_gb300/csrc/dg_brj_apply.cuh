@@ -35,15 +35,30 @@ __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
                  : "memory");
 }
 
+// How the off-diagonal product applies the dense inverse mass matrix of a
+// general element; the same sums in the same order, whichever reads them.
+//  MI_STAGED  through shared memory in the apply precision, a thread per
+//             (variable, mode): the loads overlap the neighbour gather, at the
+//             price of NM^2 values of shared memory a block
+//  MI_ROW     a thread per (variable, mode), entries from L1/L2
+//  MI_MODE    a thread per mode, each entry read once for all variables
+enum MinvForm { MI_STAGED, MI_ROW, MI_MODE };
+// the sweeps of one launch, one to six blocks an SM: staged up to 64 modes
+// (O-grid 24x48x6 P = 3 BRJ(7): FP32 3631 us by mode, 3369 staged; BF16 3495 and
+// 2359); with 125 modes a matrix is 62 KB, and 125 threads that read each entry
+// once beat 625 that read it five times (8x16x4 P = 4: FP32 1339 and 1674 us)
+constexpr MinvForm sweep_minv_form(int NM) { return NM <= 64 ? MI_STAGED : MI_MODE; }
+
 // The off-diagonal product of element e by one block of NTH threads: the
 // neighbour face values are evaluated from the neighbour's face-mode
 // coefficients (2-D sum factorisation), multiplied by the stored neighbour
 // trace Jacobians, lifted onto the face modes and multiplied by the inverse
 // mass matrix, all in the apply precision TA; emit(i, y_i) receives
 // y_e = q_e + dt_a M^-1 (...) entry by entry (i = v N_m + m).
+// MI: how a general element's dense M^-1 is applied.
 // COOP: qh is written by other blocks of the same launch, so it is read from L2.
-template <int DIM, int P, int Q, typename TA, typename TJ, bool CV, int NTH, bool COOP = false,
-          class Emit>
+template <int DIM, int P, int Q, typename TA, typename TJ, bool CV, int NTH, MinvForm MI,
+          bool COOP = false, class Emit>
 __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo* __restrict__ geo,
                                                 const double* __restrict__ minv,
                                                 const TJ* __restrict__ Jo,
@@ -66,21 +81,22 @@ __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo
     prefetch_l2(Jo + ((long long)e * 2 * DIM + threadIdx.x) * NV * NV * NF, sizeof(TJ) * NV * NV * NF);
   else if (threadIdx.x == 2 * DIM)
     prefetch_l2(q + (long long)e * NV * NM, sizeof(double) * NV * NM);
-  // general elements: M_e^-1 in the apply precision.  Up to 64 modes it is
-  // staged in shared memory, its loads issued before the gather whose phases
-  // they overlap; larger ones are read where they are used
-  constexpr bool STAGE = CV && NM <= 64;
+  // the first AHEAD values of a thread's share of M_e^-1 are loaded before the
+  // gather, whose phases they overlap, the rest after it (all of them ahead
+  // spilled the FP32 sweep at its 40 registers: 24x48x6 P = 3 3455 us, 3369 so)
+  constexpr bool STAGE = CV && MI == MI_STAGED;
   __shared__ TA sMe[STAGE ? NM * NM : 1];
-  constexpr int NME = STAGE ? (NM * NM + NTH - 1) / NTH : 1;
-  double me[NME];
-  if constexpr (STAGE) {
+  constexpr int NME = STAGE ? (NM * NM + NTH - 1) / NTH : 1, AHEAD = NME < 8 ? NME : 8;
+  double me[AHEAD];
+  auto load_minv = [&](int t0) {
     const double* Me = minv + (long long)e * NM * NM;
 #pragma unroll
-    for (int t = 0; t < NME; ++t) {
-      const int i = threadIdx.x + NTH * t;
-      me[t] = i < NM * NM ? __ldcs(Me + i) : 0.0;
+    for (int t = 0; t < AHEAD; ++t) {
+      const int i = threadIdx.x + NTH * (t0 + t);
+      me[t] = t0 + t < NME && i < NM * NM ? __ldcs(Me + i) : 0.0;
     }
-  }
+  };
+  if constexpr (STAGE) load_minv(0);
   for (int i = threadIdx.x; i < Q * N; i += blockDim.x) sB[i] = (TA)tab.B[i];
   for (int i = threadIdx.x; i < N * N; i += blockDim.x) sMi[i] = (TA)tab.Minv[i];
   // gather the neighbour's face slice (modes with m_r = vertex of its face)
@@ -107,9 +123,13 @@ __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo
   }
   if constexpr (STAGE) {
 #pragma unroll
-    for (int t = 0; t < NME; ++t) {
-      const int i = threadIdx.x + NTH * t;
-      if (i < NM * NM) sMe[i] = (TA)me[t];
+    for (int t0 = 0; t0 < NME; t0 += AHEAD) {
+      if (t0 > 0) load_minv(t0);
+#pragma unroll
+      for (int t = 0; t < AHEAD; ++t) {
+        const int i = threadIdx.x + NTH * (t0 + t);
+        if (t0 + t < NME && i < NM * NM) sMe[i] = (TA)me[t];
+      }
     }
   }
   __syncthreads();
@@ -204,11 +224,26 @@ __device__ __forceinline__ void offdiag_element(const Tables& tab, const ElemGeo
   }
   __syncthreads();
   if constexpr (CV) {
-    // dense inverse mass matrix of the element (symmetric), a thread per
-    // (variable, mode): with a thread per mode, 64 of 512 threads walked 64
-    // dependent loads while the rest waited (O-grid 12x24x6 P = 3, BF16
-    // blocks: 153 us per sweep of which the block product is 64)
+    // dense inverse mass matrix of the element (symmetric)
     const double* Me = minv + (long long)e * NM * NM;
+    if constexpr (MI == MI_MODE) {
+      for (int m = threadIdx.x; m < NM; m += blockDim.x) {
+        TA s2[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) s2[v] = (TA)0;
+        for (int kk = 0; kk < NM; ++kk) {
+          const TA mk = (TA)Me[kk * NM + m];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) s2[v] += mk * L0[v * NM + kk];
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const long long gi = ((long long)e * NV + v) * NM + m;
+          emit(v * NM + m, q[gi] + dta * (double)s2[v]);
+        }
+      }
+      return;
+    }
     for (int i = threadIdx.x; i < NV * NM; i += blockDim.x) {
       const int m = i % NM, v0 = i - m;
       TA s2 = (TA)0;

@@ -1273,7 +1273,7 @@ __global__ void __launch_bounds__(256) brj_invert_tc_kernel(float* __restrict__ 
 // ------------------------------------------------------------ apply
 // y = q - (L+U) qh = q + dt_a M^-1 sum_faces B_f^T (Jo . trace of the neighbour's qh)
 // y = q - (L+U) qh, one block of 128 threads per element
-template <int DIM, int P, int Q, typename TA, typename TJ, bool CV>
+template <int DIM, int P, int Q, typename TA, typename TJ, bool CV, MinvForm MI>
 __global__ void __launch_bounds__(128) brj_offdiag_kernel(
     const __grid_constant__ Tables tab, const ElemGeo* __restrict__ geo,
     const double* __restrict__ minv, int E, const TJ* __restrict__ Jo,
@@ -1281,8 +1281,9 @@ __global__ void __launch_bounds__(128) brj_offdiag_kernel(
     const double* __restrict__ q, double dta, double* __restrict__ y) {
   constexpr int NB = Cfg<DIM, P, Q>::NV * Cfg<DIM, P, Q>::NM;
   const int e = blockIdx.x;
-  offdiag_element<DIM, P, Q, TA, TJ, CV, 128>(tab, geo, minv, Jo, nbr, qh, q, dta, e,
-                                              [&](int i, double v) { y[(long long)e * NB + i] = v; });
+  offdiag_element<DIM, P, Q, TA, TJ, CV, 128, MI>(
+      tab, geo, minv, Jo, nbr, qh, q, dta, e,
+      [&](int i, double v) { y[(long long)e * NB + i] = v; });
 }
 
 // ------------------------------------------------------------ drivers
@@ -1382,7 +1383,25 @@ struct BRJImpl {
   template <typename TA, typename TJ, bool CV>
   static dg_status offdiag(dg_mesh_s* m, dg_precond_s* pc, const double* qh, const double* q,
                            double* y, cudaStream_t s) {
-    DG_PROF(K_BRJ_OFFDIAG, s, brj_offdiag_kernel<DIM, P, Q, TA, TJ, CV><<<m->E, 128, 0, s>>>(
+    // The dense M^-1 of general elements, with many blocks an SM: FP64 up to 64
+    // modes from L1 (O-grid 12x24x6 P = 2 BRJ(7) 962 us, staged 1018), FP32 staged
+    // below 64 modes (P = 2 283, 324 from L1); at 64 a staged matrix is 16 KB and
+    // halves the blocks an SM holds, so it pays while one wave holds all elements
+    // (P = 3, 120 elements 244 us, by mode 257; 1728: 1008 and 997; 6912: 3672 and
+    // 3497); larger ones by mode (P = 4, 512 elements: 1370, 1727 from L1).
+    constexpr int NM = C::NM;
+    if constexpr (CV && NM == 64 && std::is_same<TA, float>::value) {
+      if (m->E > 7 * 152)
+        return offdiag_form<TA, TJ, CV, MI_MODE>(m, pc, qh, q, y, s);
+    }
+    constexpr MinvForm MI =
+        NM > 64 ? MI_MODE : (std::is_same<TA, double>::value ? MI_ROW : MI_STAGED);
+    return offdiag_form<TA, TJ, CV, MI>(m, pc, qh, q, y, s);
+  }
+  template <typename TA, typename TJ, bool CV, MinvForm MI>
+  static dg_status offdiag_form(dg_mesh_s* m, dg_precond_s* pc, const double* qh, const double* q,
+                                double* y, cudaStream_t s) {
+    DG_PROF(K_BRJ_OFFDIAG, s, brj_offdiag_kernel<DIM, P, Q, TA, TJ, CV, MI><<<m->E, 128, 0, s>>>(
         m->tab, m->geo, m->minv, m->E, (const TJ*)pc->jo, pc->nbr, qh, q, pc->dt_a, y));
     DG_LAUNCHED(1);
     return DG_OK;

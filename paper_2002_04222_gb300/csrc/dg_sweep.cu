@@ -40,7 +40,7 @@ __global__ void DG_DIAG_BOUNDS(TB)
     if (nc > 0)
       prefetch_l2(blocks + (long long)e * nb * ld + (long long)c0 * ld, sizeof(TB) * (size_t)nc * ld);
   }
-  offdiag_element<DIM, P, Q, TA, TJ, CV, NTH>(tab, geo, minv, Jo, nbr, qprev, q, dta, e,
+  offdiag_element<DIM, P, Q, TA, TJ, CV, NTH, sweep_minv_form(Cfg<DIM, P, Q>::NM)>(tab, geo, minv, Jo, nbr, qprev, q, dta, e,
                                               [&](int i, double v) { sy[i] = (TA)v; });
   __syncthreads();
   diag_element<TB>(blocks, nb, ld, split, sy, part, qprev, omega, out, e);
@@ -120,7 +120,7 @@ __global__ void DG_DIAG_BOUNDS(TB)
   for (int j = 1; j < J; ++j) {
     ok = grid_meet(bar, polls) && ok;
     double* nxt = j == J - 1 ? out : (cur == qa ? qb : qa);
-    offdiag_element<DIM, P, Q, TA, TJ, CV, NTH, true>(
+    offdiag_element<DIM, P, Q, TA, TJ, CV, NTH, sweep_minv_form(Cfg<DIM, P, Q>::NM), true>(
         tab, geo, minv, Jo, nbr, cur, q, dta, e, [&](int i, double v) { sy[i] = (TA)v; });
     __syncthreads();
     diag_element<TB, true>(blocks, nb, ld, split, sy, part, cur, omega, nxt, e);
