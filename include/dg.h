@@ -432,8 +432,9 @@ long long dg_kernel_launches(void);
  * launch stream.  dg_profile_read synchronises the device and returns, per
  * kernel family, the launch count and summed device time since the previous
  * read (at most cap entries in out, *n set to the number written); dg_lift
- * counts the passes of the lift, which run inside the dg_vol kernel and take
- * their time there. */
+ * counts the passes of the lift, which run inside the dg_vol kernel: it has no
+ * launches and no time of its own.  dg_trace are the traces that a
+ * preconditioner build takes. */
 typedef struct {
   char name[24];
   long long launches;

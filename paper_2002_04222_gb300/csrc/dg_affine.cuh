@@ -1009,7 +1009,7 @@ dg_status launch_fix(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
     DG_CUDA(cudaFuncSetAttribute(vol_fix_kernel<DIM, P, Q>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm));
     // (the lift family counts the pass too: its work is in this kernel)
-    prof_end(prof_begin(K_LIFT, s), s);
+    prof_pass(K_LIFT);
     DG_PROF(K_VOL, s, vol_fix_kernel<DIM, P, Q>
             <<<(m->E + epb - 1) / epb, m->tune.vol_threads, vsm, s>>>(
         m->fix, m->phys, m->geo, m->E, a.u, a.v, a.eps, m->eface, m->faces, m->F, m->fflux, m->fexp,

@@ -6,6 +6,7 @@
 #include <cstring>
 #include <cstdio>
 #include <new>
+#include <utility>
 #include <vector>
 #include "dg_internal.h"
 #include "dg_precond.h"
@@ -18,7 +19,7 @@ long long g_launches = 0;
 static const char* kernel_names[K_COUNT] = {
     "dg_vol", "dg_face", "dg_lift", "dg_project", "dot", "multi_dot", "multi_axpy", "vector",
     "brj_weights", "brj_tracejac", "brj_block", "brj_invert", "brj_diag",
-    "brj_offdiag", "mlp_gemm", "brj_sweep", "dg_sensor"};
+    "brj_offdiag", "mlp_gemm", "brj_sweep", "dg_sensor", "dg_trace"};
 struct ProfRec {
   int id;
   cudaEvent_t a, b;
@@ -26,6 +27,7 @@ struct ProfRec {
 static bool g_prof = false;
 static std::vector<ProfRec> g_recs;
 static std::vector<cudaEvent_t> g_event_pool;
+static long long g_passes[K_COUNT];  // counted without a launch of their own
 
 static cudaEvent_t take_event() {
   if (!g_event_pool.empty()) {
@@ -51,6 +53,10 @@ int prof_begin(int id, cudaStream_t s) {
 void prof_end(int h, cudaStream_t s) {
   if (h < 0) return;
   cudaEventRecord(g_recs[h].b, s);
+}
+
+void prof_pass(int id) {
+  if (g_prof) g_passes[id]++;
 }
 
 dg_status cuda_status(cudaError_t e) {
@@ -268,6 +274,7 @@ dg_status dg_profile_read(dg_kernel_time* out, int cap, int* n) {
     g_event_pool.push_back(r.b);
   }
   g_recs.clear();
+  for (int i = 0; i < K_COUNT; ++i) cnt[i] += std::exchange(g_passes[i], 0);
   int k = 0;
   for (int i = 0; i < K_COUNT; ++i) {
     if (cnt[i] == 0) continue;

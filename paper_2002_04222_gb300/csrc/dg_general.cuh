@@ -958,7 +958,7 @@ dg_status launch_gen(dg_mesh_s* m, const EvalArgs& a, cudaStream_t s) {
   if (!a.skip_vol) {
     DG_CUDA(cudaFuncSetAttribute(vol_gen_kernel<DIM, P, Q>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm));
-    prof_end(prof_begin(K_LIFT, s), s);  // (as on axis-aligned elements)
+    prof_pass(K_LIFT);  // (as on axis-aligned elements)
     DG_PROF(K_VOL, s, vol_gen_kernel<DIM, P, Q>
             <<<(m->E + epb - 1) / epb, m->tune.vol_threads, vsm, s>>>(
         m->fix, m->phys, gg, m->eminv, m->E, a.u, a.v, a.eps, m->eface, m->faces, m->F, m->fflux,

@@ -174,10 +174,11 @@ extern long long g_launches;
 enum KernelId {
   K_VOL, K_FACE, K_LIFT, K_PROJECT, K_DOT, K_MULTIDOT, K_MULTIAXPY, K_VEC,
   K_BRJ_WEIGHTS, K_BRJ_TRACEJAC, K_BRJ_BLOCK, K_BRJ_INVERT, K_BRJ_DIAG,
-  K_BRJ_OFFDIAG, K_MLP, K_BRJ_SWEEP, K_SENSOR, K_COUNT
+  K_BRJ_OFFDIAG, K_MLP, K_BRJ_SWEEP, K_SENSOR, K_TRACE, K_COUNT
 };
 int prof_begin(int id, cudaStream_t s);
 void prof_end(int handle, cudaStream_t s);
+void prof_pass(int id);  // a pass that runs inside another kernel: counted, no time
 bool profiling_on();
 #define DG_PROF(id, stream, ...)                    \
   do {                                              \

@@ -412,7 +412,7 @@ static dg_status run_traces_g(dg_mesh_s* m, const double* u, cudaStream_t s) {
   const size_t sm = sizeof(double) * C::VOL_SM;
   DG_CUDA(cudaFuncSetAttribute(trace_kernel<DIM, P, Q, CV>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  DG_PROF(K_VOL, s, trace_kernel<DIM, P, Q, CV><<<(m->E + C::EPB - 1) / C::EPB, C::NT, sm, s>>>(
+  DG_PROF(K_TRACE, s, trace_kernel<DIM, P, Q, CV><<<(m->E + C::EPB - 1) / C::EPB, C::NT, sm, s>>>(
       m->tab, m->geo, gen_geo(m), m->E, u, m->tbuf));
   DG_LAUNCHED(1);
   return DG_OK;
