@@ -25,6 +25,12 @@ __device__ __forceinline__ void mode_coords(int m, int* mc) {
   X(2, 1, 3) X(2, 2, 3) X(2, 2, 4) X(2, 3, 5) X(2, 4, 6) X(2, 5, 7) X(2, 6, 8) X(3, 1, 3) \
   X(3, 2, 4) X(3, 2, 5) X(3, 3, 5) X(3, 3, 6) X(3, 4, 6) X(3, 4, 8)
 
+// FP64 blocks on general elements are offered up to P = 2 (dg_precond_build)
+template <int D, int P, int Q, typename T>
+constexpr bool has_curved_blocks() {
+  return has_curved<D, P, Q>() && !(sizeof(T) == 8 && P > 2);
+}
+
 // Hint that brings the 16-byte-aligned interior of [p, p + bytes) of global
 // memory toward L2 (bulk prefetch: no registers, no shared memory, no wait).
 __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {

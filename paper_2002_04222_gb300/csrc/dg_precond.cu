@@ -1459,7 +1459,7 @@ template <int D, int P, int Q, typename T>
 static dg_status build_dispatch(dg_mesh_s* m, dg_precond_s* pc, const double* u, double t,
                                 double dta, cudaStream_t s) {
   if (!m->curved) return BRJImpl<D, P, Q>::template build<T, false>(m, pc, u, t, dta, s);
-  if constexpr (has_curved<D, P, Q>())
+  if constexpr (has_curved_blocks<D, P, Q, T>())
     return BRJImpl<D, P, Q>::template build<T, true>(m, pc, u, t, dta, s);
   return DG_ERR_UNSUPPORTED;
 }
@@ -1468,7 +1468,7 @@ template <int D, int P, int Q, typename TA>
 static dg_status offdiag_dispatch(dg_mesh_s* m, dg_precond_s* pc, const double* qh,
                                   const double* q, double* y, cudaStream_t s) {
   if (!m->curved) return BRJImpl<D, P, Q>::template offdiag<TA, TA, false>(m, pc, qh, q, y, s);
-  if constexpr (has_curved<D, P, Q>())
+  if constexpr (has_curved_blocks<D, P, Q, TA>())
     return BRJImpl<D, P, Q>::template offdiag<TA, TA, true>(m, pc, qh, q, y, s);
   return DG_ERR_UNSUPPORTED;
 }

@@ -13,7 +13,6 @@ struct Cfg {
   static constexpr int NM = DIM == 2 ? N * N : N * N * N;
   static constexpr int NQ = DIM == 2 ? Q * Q : Q * Q * Q;
   static constexpr int NF = DIM == 2 ? Q : Q * Q;
-  static constexpr int NFACE = 2 * DIM;
   static constexpr int NFLD = 1 + DIM;
   static constexpr int NT = 256;
   static constexpr int EPB = DIM == 2 ? (NT / NQ > 0 ? NT / NQ : 1) : 1;
@@ -74,19 +73,12 @@ __device__ __forceinline__ void stage_tables(const Tables& tab, double* s) {
   for (int i = threadIdx.x; i < N * N; i += blockDim.x) s[Q * N + Q * Q + 2 * Q + i] = tab.Minv[i];
 }
 
-// Coordinates (q0, q1, q2) of Gauss-grid point q and face-point index of the
-// face normal to direction r.
+// Coordinates (q0, q1, q2) of Gauss-grid point q.
 template <int DIM, int Q>
 __device__ __forceinline__ void grid_coords(int q, int* c) {
   c[0] = q % Q;
   c[1] = (q / Q) % Q;
   c[2] = DIM == 3 ? q / (Q * Q) : 0;
-}
-template <int DIM, int Q>
-__device__ __forceinline__ int face_point(const int* c, int r) {
-  if (DIM == 2) return c[1 - r];
-  const int t0 = r == 0 ? 1 : 0, t1 = r == 2 ? 1 : 2;
-  return c[t0] + Q * c[t1];
 }
 
 }  // namespace dg

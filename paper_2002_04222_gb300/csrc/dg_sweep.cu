@@ -173,7 +173,7 @@ static dg_status coop_launch(dg_precond_s* pc, const double* q, double* out, cud
 template <int D, int P, int Q, typename TB>
 static dg_status coop_dispatch_t(dg_precond_s* pc, const double* q, double* out, cudaStream_t s) {
   if (!pc->mesh->curved) return coop_launch<D, P, Q, TB, false>(pc, q, out, s);
-  if constexpr (has_curved<D, P, Q>()) return coop_launch<D, P, Q, TB, true>(pc, q, out, s);
+  if constexpr (has_curved_blocks<D, P, Q, TB>()) return coop_launch<D, P, Q, TB, true>(pc, q, out, s);
   return DG_ERR_UNSUPPORTED;
 }
 
@@ -194,7 +194,7 @@ template <int D, int P, int Q, typename TB>
 static dg_status sweep_dispatch(dg_precond_s* pc, const double* qprev, const double* q,
                                 double* out, cudaStream_t s) {
   if (!pc->mesh->curved) return sweep_launch<D, P, Q, TB, false>(pc, qprev, q, out, s);
-  if constexpr (has_curved<D, P, Q>()) return sweep_launch<D, P, Q, TB, true>(pc, qprev, q, out, s);
+  if constexpr (has_curved_blocks<D, P, Q, TB>()) return sweep_launch<D, P, Q, TB, true>(pc, qprev, q, out, s);
   return DG_ERR_UNSUPPORTED;
 }
 
