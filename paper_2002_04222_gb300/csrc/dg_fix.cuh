@@ -28,7 +28,11 @@ namespace dg {
 typedef long long i64;
 typedef unsigned long long u64;
 
-constexpr int FIX_EMIN = 200;   // exponents below (2^-823) count as this: smaller inputs become 0
+// Exponents below this (2^-783) count as this, so that smaller inputs become 0.
+// The last conversion of M^-1 B^T W G has a scale of up to 3 x 59 + 60 powers of
+// two less (every stage's input shifted up), which has to stay a normal
+// double's: fix_to_double adds to the exponent field without a look at its range.
+constexpr int FIX_EMIN = 240;
 constexpr int FIX_EBAD = 2010;  // largest exponent held; from here on (2^987) the result is NaN
 
 // 32 x 32 -> 64-bit product, to be accumulated with +=: the product in PTX and

@@ -9,11 +9,11 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2002_04222_gb300", "csrc")
 
 
-def run_host(tmp_path, body, lines):
+def run_host(tmp_path, body, lines, extra=""):
     """stdout of a host program whose main() reads the lines' numbers."""
     from paper_2002_04222_gb300.build import nvcc
     src, exe = tmp_path / "probe.cu", tmp_path / "probe"
-    src.write_text('#include <cstdio>\n#include "dg_fix.cuh"\nusing namespace dg;\n'
+    src.write_text('#include <cstdio>\n#include "dg_fix.cuh"\n' + extra + "using namespace dg;\n"
                    "int main() {\n" + body + "\nreturn 0; }\n")
     subprocess.run([nvcc(), "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a",
                     "--expt-relaxed-constexpr", "-I", CSRC, str(src), "-o", str(exe)], check=True)
@@ -65,3 +65,19 @@ def test_products_round_alike_on_both_signs(tmp_path):
         assert 0 <= sign * x <= exact + 1 and exact - sign * x < 3, (v, r, x)
         by.setdefault((abs(v), abs(r)), set()).add(sign * x)
     assert all(len(s) == 1 for s in by.values())
+
+
+def test_the_smallest_scale_is_a_normal_double(tmp_path):
+    """One unit of M^-1 B^T W G at the smallest shared exponent, every stage's
+    input shifted up as far as it goes (59 places) and two bits kept below the
+    last stage's unit, is 2^-1022 at least: fix_to_double has no subnormals (a
+    smaller scale borrowed from the sign bit and came out near 2^1000)."""
+    inst = ([(2, p, q) for p, q in ((1, 3), (2, 3), (2, 4), (3, 5), (4, 6), (5, 7), (6, 8))]
+            + [(3, p, q) for p, q in ((1, 3), (2, 4), (2, 5), (3, 5), (3, 6), (4, 6), (4, 8))])
+    got = run_host(tmp_path, 'int d, P, Q; FixTab f; '
+                             'while (scanf("%d %d %d", &d, &P, &Q) == 3) { build_fix_tables(P, Q, f); '
+                             'printf("%d\\n", FIX_EMIN - 1022 - 58 - 2 - 59 * d + f.eDh + d * f.eA); }',
+                   [f"{d} {p} {q}" for d, p, q in inst], extra='#include "dg_fixtab.cu"\n')
+    assert len(got) == len(inst)
+    for i, g in zip(inst, got):
+        assert int(g) >= -1022, (i, g)
