@@ -34,6 +34,7 @@
 #include "dg_sumfact.cuh"
 #include "dg_tc.cuh"
 #include "dg_brj_apply.cuh"
+#include "dg_pairs.cuh"
 
 namespace dg {
 
@@ -446,27 +447,6 @@ __global__ void __launch_bounds__(128) brj_tracejac_gen_kernel(
 // q0 per (j,a) accumulated by the types of direction 1, then q1.  The own-side
 // trace term adds, on each face, the face-slice modes (vertex mode across the
 // face) contracted over the two (one) tangential face-point directions.
-template <int N, typename T>
-__device__ __forceinline__ T fp64_row(const double* m, const T* x, int str) {
-  double s = 0.0;
-#pragma unroll
-  for (int k = 0; k < N; ++k) s += m[k] * (double)x[k * str];
-  return (T)s;
-}
-template <typename T>
-__device__ __forceinline__ T fp64_scaled(double sc, T x, double add) {
-  return (T)__dadd_rn(__dmul_rn(sc, (double)x), add);
-}
-// out of line for the values that float pairs cannot decide (PairSum): inlined
-// there, the FP64 pipe is as busy as without the pairs
-template <int N, typename T>
-__device__ __noinline__ T fp64_row_call(const double* m, const T* x, int str) {
-  return fp64_row<N>(m, x, str);
-}
-__device__ __noinline__ float fp64_scaled_call(double sc, float x, double add) {
-  return fp64_scaled(sc, x, add);
-}
-
 // shared-memory layout of the block assembly (sizes in T)
 template <int DIM, int P, int Q, typename T>
 struct BlockSmem {
@@ -485,39 +465,6 @@ struct BlockSmem {
   // 10^3 blocks 17.2 ms against 16.4 with the former layouts)
   static constexpr bool T1_IN_Y = DIM == 3 && 4 * Q * N2 + T1SZ <= NM * XS;
   static constexpr int SCRATCH = NQ * DIM * (DIM + 1) + (T1_IN_Y ? 0 : T1SZ) + T2SZ;  // sW, T1, T2
-};
-
-// FP32 results of FP64 arithmetic without the FP64 pipe.  A sum of products
-// m_k x_k (m_k doubles, x_k floats) is formed in float pairs (error below 2^-42
-// of the terms' magnitudes) and rounded; where it lies too close to a rounding
-// boundary to tell on which side the FP64 sum falls, near() says so and the
-// caller takes the FP64 form, so that the result is FP64's bit for bit.  The
-// mass-matrix step of a P = 3 block is 49,000 FP64 multiply-adds, 25 blocks per
-// element, on a pipe that retires two per clock.  Entries that cancel to
-// rounding noise cannot be told and keep FP64 (6^3 elements, P = 3: 1.30 ms of
-// assembly with FP64 and the former shared-memory layouts, 0.99 with both).
-struct PairSum {
-  float s = 0.f, c = 0.f, big = 0.f;
-  __device__ __forceinline__ void add(float mh, float ml, float x) {
-    const float p = __fmul_rn(mh, x);
-    const float e = __fmaf_rn(ml, x, __fmaf_rn(mh, x, -p));
-    const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
-    const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b));
-    s = t;
-    c = __fadd_rn(c, __fadd_rn(r, e));
-    big += fabsf(p);
-  }
-  __device__ __forceinline__ float value() const { return __fadd_rn(s, c); }
-  // the pair within 2^-42 of the terms of a boundary between two floats, or
-  // out of the range where that is told apart from the value's own exponent
-  __device__ __forceinline__ bool near(float v) const {
-    const int b = __float_as_int(v), E = b & 0x7f800000;
-    const float half = __int_as_float(E - (24 << 23));  // half a unit of v
-    const float left = fabsf(__fsub_rn(c, __fsub_rn(v, s)));
-    return big != 0.f && (E < (60 << 23) || E > (250 << 23) ||
-                          (b & 0x7fffff) == 0 ||
-                          !(half - left > big * 2.3e-13f));
-  }
 };
 
 // blocks per SM: FP32 up to P = 3 three; the smallest elements' blocks are a few
@@ -827,11 +774,7 @@ __global__ void __launch_bounds__(256, block_residency<DIM, P, T>()) brj_block_k
       const T* x = src + col * XS + base;
       T val;
       if constexpr (PAIRS) {
-        PairSum ps;
-#pragma unroll
-        for (int kk = 0; kk < N; ++kk) ps.add(sMh[mc[ax] * N + kk], sMl[mc[ax] * N + kk], x[kk * str]);
-        val = ps.value();
-        if (ps.near(val)) val = fp64_row_call<N>(sMi + mc[ax] * N, x, str);
+        val = pair_row<N>(sMh + mc[ax] * N, sMl + mc[ax] * N, sMi + mc[ax] * N, x, str);
       } else {
         val = CALL ? fp64_row_call<N>(sMi + mc[ax] * N, x, str) : fp64_row<N>(sMi + mc[ax] * N, x, str);
       }
@@ -852,10 +795,7 @@ __global__ void __launch_bounds__(256, block_residency<DIM, P, T>()) brj_block_k
     const double one = k == l && m == n ? 1.0 : 0.0;
     T v;
     if constexpr (PAIRS) {
-      PairSum ps;
-      ps.add(sh, sl, x);
-      v = ps.value();
-      if (one != 0.0 || ps.near(v)) v = fp64_scaled_call(sc, x, one);
+      v = pair_scaled(sh, sl, sc, x, one);
     } else {
       v = fp64_scaled(sc, x, one);
     }
