@@ -756,7 +756,10 @@ static dg_status gmres_impl(dg_mesh_s* m, dg_precond_s* p, const double* u, cons
         const double* zk = vk;
         if (p) {
           double* zz = Z + (size_t)k * n;
-          if (p->use_graphs && !profiling_on())
+          // (the handle's own graphs: the fused sweeps replayed, 8x8 P = 2 FP64
+          // 124 us an iteration, one launch 128; the two-kernel ones where the
+          // mesh is large, else they lose: 6^3 P = 3 FP64 1417 and 896)
+          if (p->use_graphs && (p->fused || !p->coop) && !profiling_on())
             DG_TRY(precond_apply_impl(p, vk, zz, s));
           else
             DG_TRY(precond_solver_apply(p, vk, zz, false, s));

@@ -1483,7 +1483,8 @@ dg_status precond_sweeps(dg_precond_s* pc, const double* q, double* out, cudaStr
 //  - Launched one by one, the two-kernel sweeps pay 2J-1 gaps: one launch wins
 //    (2-D P = 2 FP64 E = 64 43 / 66, E = 900 86 / 112; 3-D P = 2 FP32 E = 64
 //    73 / 105) until a block takes longer than its gap: 3-D P = 3, curved, FP32
-//    E = 800 547 / 526, fused 514.  From 320 unknowns an element on, never.
+//    E = 800 547 / 526, fused 514.  From 320 unknowns an element on, never (FP64
+//    E = 216 747, fused 692; E = 512 the one measured exception, 1008 and 1071).
 //  - The fused sweeps have half the gaps: against them one launch wins up to
 //    100 unknowns an element (2-D P = 2 FP64 E = 64 44 / 54, P = 4 FP32 E = 900
 //    81 / 82; not BF16 blocks of 16 unknowns: 60 / 56), beyond that while an SM
