@@ -79,3 +79,22 @@ def test_solves_on_both_sides_of_the_cluster_limit(dgl, nx, ny):
     err = torch.linalg.norm(b - ax).item()
     bound = 1e-4 * torch.linalg.norm(b).item() + 1e-6 * torch.linalg.norm(ax).item()
     assert err < bound, (err, bound)
+
+
+@pytest.mark.parametrize("nx,ny", [(16, 64), (27, 38)])
+def test_a_full_basis_on_both_sides_of_the_cluster_limit(dgl, nx, ny):
+    """16,384 unknowns and 16,416 with a basis of 64 vectors, none converged
+    before it is full: the residual that the Hessenberg matrix tells (orthonormal
+    vectors) is the true one, to the finite-difference product's 1e-6."""
+    c = w.poiseuille_case(1, nx=nx, ny=ny)
+    m = dgl.Mesh.from_case(c)
+    u = m.project()
+    g = torch.Generator(device="cuda").manual_seed(1)
+    b = torch.randn(u.shape, dtype=torch.float64, device="cuda", generator=g)
+    r = m.residual(u)
+    dta = 0.05
+    x, st = m.gmres(u, r, b, 0.0, dta, restart=64, max_cycles=1, rtol=1e-14)
+    assert st["iters"] == 64 and 0.0 < st["res"] < st["res0"]
+    ax = m.jvp(u, r, x, 0.0, 1.0, -dta)
+    err = abs(torch.linalg.norm(b - ax).item() - st["res"])
+    assert err < 1e-6 * torch.linalg.norm(ax).item() + 1e-10 * st["res0"], (err, st)
