@@ -178,12 +178,13 @@ class Clocks:
 
 
 # ------------------------------------------------------------------ work model
-def residual_flops_per_elem(P, Q, d=3):
+def residual_fp64_slots_per_elem(P, Q, d=3):
     """FP64 work of one residual per element, as the two kernels implement it:
     the pointwise fluxes (the contractions run in fixed point on the integer
     pipe; the lift is part of the volume kernel).  Counted in FP64 instructions
     per volume point and face point (ncu, constant viscosity, Roe), each as the
-    2 flops of the FMA slot it takes in the pipe."""
+    2 flops of the FMA slot it takes in the pipe: a measure of how full the pipe
+    is, not of the method's flops."""
     c_F, c_T = 2 * 120, 2 * 249
     return {"dg_vol": c_F * Q ** 3, "dg_face": d * Q ** 2 * c_T}   # d faces per element
 
@@ -191,7 +192,7 @@ def residual_flops_per_elem(P, Q, d=3):
 def kernel_work(name, launches, E, nb, prec_bytes, P, Q, d=3):
     """(bound, algorithmic units per launch, unit) of a kernel family.  The
     residual kernels' flop counts are those of the 3-D kernels."""
-    f = residual_flops_per_elem(P, Q)
+    f = residual_fp64_slots_per_elem(P, Q)
     if name in f:
         return ("alu", f[name] * E, "flop") if d == 3 else (None, None, None)
     if name == "brj_diag":
@@ -418,12 +419,14 @@ def run_ours(args, rank, world):
     e1.record(stream)
     torch.cuda.synchronize()
     res_ms = e0.elapsed_time(e1) / nres
-    # the residual's roofline: the FP64 work of its pointwise fluxes over the
-    # measured FP64 FMA throughput of this GPU, taken in this run
-    rflops = sum(residual_flops_per_elem(wl["P"], wl["Q"]).values()) * E
+    # the residual's share of the FP64 pipe: the instruction slots of its
+    # pointwise fluxes (2 flops each) over the measured FP64 FMA throughput of
+    # this GPU, taken in this run
+    rflops = sum(residual_fp64_slots_per_elem(wl["P"], wl["Q"]).values()) * E
     res_roof = {"bound": "alu", "achieved": rflops / (res_ms / 1e3) / 1e12, "peak": fp64_peak,
                 "unit": "TFLOP/s", "frac": rflops / (res_ms / 1e3) / 1e12 / fp64_peak,
-                "flops_per_launch": rflops, "avg_ms": res_ms,
+                "slot_flops_per_launch": rflops, "avg_ms": res_ms,
+                "counts": "2 flops per FP64 instruction slot of the pointwise fluxes",
                 "peak_source": "measured in this run: dg_peak_fp64 (FP64 FMA chains at full "
                                "occupancy, CUDA events)"}
     if dim != 3:
@@ -431,7 +434,7 @@ def run_ours(args, rank, world):
                     "avg_ms": res_ms, "note": "flop counts are those of the 3-D kernels"}
     for kname in ("dg_vol", "dg_face"):
         if kname in prof and not cyl and dim == 3:
-            kf = residual_flops_per_elem(wl["P"], wl["Q"])[kname] * E
+            kf = residual_fp64_slots_per_elem(wl["P"], wl["Q"])[kname] * E
             kms = prof[kname][1] / prof[kname][0]
             res_roof[kname] = {"avg_ms": round(kms, 4),
                                "frac": round(kf / (kms / 1e3) / 1e12 / fp64_peak, 3)}
@@ -524,7 +527,7 @@ def run_ours(args, rank, world):
         "gpu_launches": launches,
         "clocks": clk,
         "roofline": roof,
-        "residual_roofline": res_roof,
+        "residual_fp64_pipe": res_roof,
         "variants": variants,
         "kernels": kernels,
         "e2e": e2e,

@@ -6,10 +6,10 @@
 //                    both (D_j^T, J^T), M^-1 B^T, and the residual's or the
 //                    Jacobian-free product's epilogue.
 // All contractions run in 64-bit fixed point (dg_fix.cuh); FP64 remains for
-// the pointwise fluxes, which bound both kernels: 216 volume points of about
-// 110 FP64 instructions and 108 face points of about 240 per element at P = 3
-// against about 55,000 multiply-adds of contractions, which took 60% of the
-// FP64 pipe's time when they ran there.
+// the pointwise fluxes, which bound both kernels: 216 volume points of 120 FP64
+// instructions and 108 face points of 249 per element at P = 3 (ncu) against
+// about 70,000 multiply-adds of contractions, which took 60% of the FP64 pipe's
+// time when they ran there.
 //
 // With H~_r = (2/h_r) H_r, w the 1-D weights and M1 the 1-D mass matrix, the
 // metric cancels between M^-1 and the integrals:
@@ -266,7 +266,8 @@ __device__ __noinline__ void own_values(const FixTab& ft, const Info* info, cons
 // point in the flux.  FPB faces per block.  80 registers: the FP64 pipe waits
 // on the other phases unless several blocks share an SM, and the few spilled
 // values cost less (16^3 P = 3: 262 us at 128 registers, 245 at 96, 236 at 80;
-// FP64 floor 184 us at 16 clocks per warp instruction).
+// FP64 floor 184 us at 16 clocks per warp instruction; the 2-D instances were
+// not timed with other limits).
 template <int DIM, int P, int Q>
 __global__ void __maxnreg__(80) face_fix_kernel(
     const __grid_constant__ FixTab ft, const __grid_constant__ Tables tab,

@@ -27,8 +27,11 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // registers, warps reduce eight sums at once (9 FP64 additions instead of 40:
 // the pipe retires one warp addition per 16 clocks), the blocks' sums meet in
 // distributed shared memory in rank order.  On the 8x8 P = 2 vortex (2304
-// unknowns) the 9 launches of the tail took about 40 us.  From here on the
-// grid-wide kernels below win (8 SMs of FP64 against all).
+// unknowns) the 9 launches of the tail took about 40 us.  Every k up to the
+// largest restart gains up to this n (us per tail in a graph, one cluster / the
+// grid-wide kernels: n = 2304 k = 8 16 / 39, k = 30 38 / 100; n = 16,384 k = 8
+// 31 / 40, k = 30 94 / 101, k = 64 178 / 182; a dot product 4.1 / 6.0); beyond it
+// the cluster's 8 SMs of FP64 fall behind and the entries leave the registers.
 namespace cg = cooperative_groups;
 constexpr int CL = 8, CT = 256, CR = 8;
 constexpr long long SMALL_N = (long long)CL * CT * CR;

@@ -1,7 +1,7 @@
 // 64-bit fixed-point arithmetic of the residual's tensor contractions.
 //
 // Why: the FP64 pipe of sm_103a retires about 2 fused multiply-adds per clock
-// and SM, the integer pipe about 55 32x32+64-bit multiply-adds (both measured
+// and SM, the integer pipe about 28 32x32+64-bit multiply-adds (both measured
 // with independent chains at full occupancy).  A contraction with a constant
 // 1-D table needs no floating point: with the inputs of one element and
 // variable scaled to their largest exponent (|x| <= 2^60) and the table to
@@ -35,11 +35,7 @@ typedef unsigned long long u64;
 constexpr int FIX_EMIN = 240;
 constexpr int FIX_EBAD = 2010;  // largest exponent held; from here on (2^987) the result is NaN
 
-// 32 x 32 -> 64-bit product, to be accumulated with +=: the product in PTX and
-// the sum in C become one IMAD.WIDE with accumulator.  (From a C product the
-// compiler sign-extends the table entries once and multiplies 64 by 64 bits;
-// from PTX multiply-adds it splits half of them into product and sum: 61
-// against 35 instructions per 36 multiply-adds.)
+// 32 x 32 -> 64-bit product, to be accumulated with +=
 DG_HD i64 mul_wide(int a, int b) {
 #ifdef __CUDA_ARCH__
   i64 d;

@@ -96,8 +96,8 @@ __device__ void sensor_element(const SensorTab& st, const Phys& ph,
   avf[e] = ph.av_mu0 * S * h / (double)P;
 }
 
-// The factor of every element at u alone (dg_av_factor); the residual
-// computes it inside the volume kernel.  One warp per element.
+// The factor of every element at u (dg_av_factor, and before the face kernel of
+// a residual with shock capturing).  One warp per element.
 constexpr int SENSOR_WARPS = 8;
 template <int DIM, int P, int Q, bool CV>
 __global__ void __launch_bounds__(32 * SENSOR_WARPS) sensor_kernel(
